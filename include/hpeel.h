@@ -72,7 +72,10 @@ typedef struct hpeel_stats {
                                round (the frontiers F_1, F_2, ...) */
     uint64_t hinge_moves;   /* peeled edges whose first claim came from a
                                vertex other than the hinge (a vertex of
-                               smaller position claimed later in the round) */
+                               smaller position claimed later in the round);
+                               0 where a round's claims are all in before its
+                               layer is listed: sorted rounds, and graphs of
+                               up to about 131,000 edges peeled in one launch */
     uint32_t async_status;  /* the *_async calls: 1 done (outputs written),
                                2 no seed peeled (builds), 3 device check
                                failed (device_err holds the code), 4 more
@@ -101,7 +104,11 @@ typedef struct hpeel_stats {
  *                       device (a CUDA graph whose while node repeats the
  *                       round kernel until a layer is empty); 1: the host
  *                       launches every round and reads the round's outcome
- *                       back before the next.
+ *                       back before the next.  With 0, a graph of up to
+ *                       131,072 edges that fits the shared memory of one
+ *                       thread-block cluster (and lies below
+ *                       bucket_min_vertices) runs its whole path in one
+ *                       launch; 1 keeps such a graph on the general path too.
  *   bucket_sub_shift    log2 of the vertices one block accumulates in shared
  *                       memory in the L2-blocked build (0 = automatic:
  *                       min(13, bucket_shift - 9); at most 14).
@@ -247,7 +254,8 @@ hpeel_status hpeel_peel_general(const uint32_t *d_edges, uint64_t n, uint64_t m,
  * The graph is built on the first call with a given set of pointers and
  * sizes and replayed by later calls with the same set (keep the workspace and
  * the output buffers to reuse it; the inputs' contents may change between
- * calls).  Returns HPEEL_OK once enqueued; errors found on the host:
+ * calls); a small graph (see the tuning's host_round_loop) is one kernel
+ * launch instead.  Returns HPEEL_OK once enqueued; errors found on the host:
  * HPEEL_ERR_INVALID_ARG, HPEEL_ERR_WORKSPACE_TOO_SMALL, HPEEL_ERR_CUDA.  When
  * stream is being captured (cudaStreamBeginCapture), the peel's nodes join
  * the caller's graph at the capture position instead.
@@ -360,7 +368,8 @@ hpeel_status hpeel_mphf_build(const uint64_t *d_keys, uint64_t n, uint64_t seed,
  *   No canonical order output.
  * The graph is built on the first call with a given set of pointers and
  * sizes and replayed by later calls with the same set (keep the workspace
- * and the output buffers to reuse it).  Returns HPEEL_OK once enqueued;
+ * and the output buffers to reuse it); a small key set (see the tuning's
+ * host_round_loop) with max_tries of at most 64 is one kernel launch instead.  Returns HPEEL_OK once enqueued;
  * errors: HPEEL_ERR_INVALID_ARG, HPEEL_ERR_WORKSPACE_TOO_SMALL, HPEEL_ERR_CUDA.
  * When stream is being captured (cudaStreamBeginCapture), the build's nodes
  * join the caller's graph at the capture position instead.

@@ -175,6 +175,15 @@ MphfLayout mphf_layout(uint64_t n, uint32_t gamma_milli) {
     return p;
 }
 
+// Where the kernel of a host-decided small call writes its stats.
+hpeel_stats *pinned_stats() {
+    thread_local hpeel_stats *p = nullptr;
+    if (!p) {
+        if (cudaMallocHost((void **)&p, sizeof(hpeel_stats)) != cudaSuccess) p = nullptr;
+    }
+    return p;
+}
+
 struct PeelOut {
     uint32_t rounds;
     uint64_t n_peeled;
@@ -199,6 +208,62 @@ struct PeelIO {
     bool host_loop = false;     // launch every round from the host, whatever the tuning
     bool random_rounds = false; // no round in sorted form
 };
+
+// Graphs that fit the shared memory of one thread-block cluster are peeled
+// (and solved) in one launch of small.cu -- at n = 1e3 and n = 1e5 alike the
+// general path spends 12 us per round on launches and trips to L2.  Not when
+// the tuning asks for the bucketed build (its threshold lies below m) or for
+// the host's round loop.  mode 0: peel, 1: MPHF, 2: static function.
+bool small_route(int mode, const PeelLayout &lay, uint64_t n, uint64_t m, uint32_t r, bool general,
+                 char *peel_ws, SmallArgs *a, SmallLaunch *k) {
+    if (lay.bucketed || tuning().host_round_loop) return false;
+    if (!small_plan(mode, n, m, r, general, a, k)) return false;
+    a->wide = reinterpret_cast<unsigned long long *>(peel_ws + lay.state);
+    return true;
+}
+
+// A small MPHF or static-function build whose outcome the host reads: launches
+// of at most kSmallTries seeds each, the last one's stats in *st.
+hpeel_status run_small_build(const Launch &L, const SmallLaunch &k, SmallArgs a, uint32_t max_tries,
+                             hpeel_stats *st) {
+    hpeel_stats *ps = pinned_stats();
+    if (!ps) return fail(HPEEL_ERR_CUDA, "cudaMallocHost of the stats read-back failed");
+    a.stats = ps;
+    const uint64_t seed = a.seed;
+    for (uint32_t done = 0; done < max_tries; done += kSmallTries) {
+        a.seed = seed + done;
+        a.max_tries = std::min(kSmallTries, max_tries - done);
+        {
+            ProfScope ps_(L, "small_build");
+            launch_small(L, k, a);
+        }
+        HP_TRY(check_launch("small build"));
+        HP_CUDA(cudaStreamSynchronize(L.stream));
+        prof_flush();
+        *st = *ps;
+        st->attempts += done;
+        if (st->async_status != kAsyncRetriesExhausted || max_tries - done <= kSmallTries) break;
+    }
+    return HPEEL_OK;
+}
+
+// The status and host stats of a small build.
+hpeel_status small_build_outcome(const hpeel_stats &st, uint64_t seed, uint32_t max_tries,
+                                 hpeel_stats *h_stats) {
+    if (h_stats) {
+        *h_stats = st;
+        h_stats->async_status = 0;
+    }
+    if (st.device_err == kDevBadValue)
+        return fail(HPEEL_ERR_DEVICE_CHECK, "a value is not below sigma (device code %u)",
+                    st.device_err);
+    if (st.device_err)
+        return fail(HPEEL_ERR_DEVICE_CHECK, "device check failed with code %u", st.device_err);
+    if (st.async_status != kAsyncPeeled)
+        return fail(HPEEL_ERR_RETRIES_EXHAUSTED, "2-core non-empty for seeds %llu..%llu",
+                    (unsigned long long)seed, (unsigned long long)(seed + max_tries - 1));
+    return HPEEL_OK;
+}
 
 // Executable graphs of the round loop, cached by their parameters: round 0,
 // then a while node whose body is one round kernel.  The round kernel's last
@@ -1160,6 +1225,37 @@ hpeel_status peel_entry(bool general, const uint32_t *d_edges, uint64_t n, uint6
     const size_t need = peel_layout(n, m, r, general).total;
     if (ws_bytes < need)
         return fail(HPEEL_ERR_WORKSPACE_TOO_SMALL, "workspace %zu < %zu bytes", ws_bytes, need);
+    SmallArgs sa{};
+    SmallLaunch sk{};
+    if (small_route(0, peel_layout(n, m, r, general), n, m, r, general, (char *)d_ws, &sa, &sk)) {
+        hpeel_stats *ps = pinned_stats();
+        if (!ps) return fail(HPEEL_ERR_CUDA, "cudaMallocHost of the stats read-back failed");
+        sa.edges = d_edges;
+        sa.order = d_order;
+        sa.claim = d_claim;
+        sa.layer_off = d_layer_off;
+        sa.max_layers = max_layers;
+        sa.stats = ps;
+        {
+            ProfScope prof(L, "small_peel");
+            launch_small(L, sk, sa);
+        }
+        HP_TRY(check_launch("small peel"));
+        HP_CUDA(cudaStreamSynchronize(L.stream));
+        prof_flush();
+        if (ps->device_err)
+            return fail(HPEEL_ERR_DEVICE_CHECK, "device check failed with code %u", ps->device_err);
+        if (d_layer_off && ps->rounds > max_layers)
+            return fail(HPEEL_ERR_CAPACITY, "%u rounds > max_layers %u", ps->rounds, max_layers);
+        if (h_stats) {
+            h_stats->n_peeled = ps->n_peeled;
+            h_stats->rounds = ps->rounds;
+            h_stats->core_nonempty = ps->core_nonempty;
+            h_stats->first_layer = ps->first_layer;
+            h_stats->frontier = ps->frontier;
+        }
+        return HPEEL_OK;
+    }
     PeelOut po{};
     PeelIO io;
     io.edges = d_edges;
@@ -1246,6 +1342,18 @@ hpeel_status peel_async_entry(bool general, const uint32_t *d_edges, uint64_t n,
                     d_layer_off, max_layers, d_stats, (char *)d_ws, L.sms};
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     HP_CUDA(cudaStreamIsCapturing(L.stream, &cs));
+    SmallArgs sa{};
+    SmallLaunch sk{};
+    if (small_route(0, peel_layout(n, m, r, general), n, m, r, general, (char *)d_ws, &sa, &sk)) {
+        sa.edges = d_edges;
+        sa.order = d_order;
+        sa.claim = d_claim;
+        sa.layer_off = d_layer_off;
+        sa.max_layers = max_layers;
+        sa.stats = d_stats;
+        launch_small(L, sk, sa);
+        return check_launch("small peel");
+    }
     if (cs == cudaStreamCaptureStatusActive) {
         // the caller is capturing: the peel's nodes join the caller's graph
         std::lock_guard<std::mutex> lk(g_graph_mu);
@@ -1319,6 +1427,19 @@ hpeel_status hpeel_mphf_build(const uint64_t *d_keys, uint64_t n, uint64_t seed,
                     lay.total);
     char *ws = (char *)d_ws;
     const FastMod fm = make_fastmod(m / 3);
+    SmallArgs sa{};
+    SmallLaunch sk{};
+    if (small_route(1, peel_layout(n, m, 3), n, m, 3, false, ws + lay.peel, &sa, &sk)) {
+        sa.keys = d_keys;
+        sa.fm = fm;
+        sa.seed = seed;
+        sa.order = d_order;
+        sa.G = d_G;
+        sa.D = d_rank_dir;
+        hpeel_stats st{};
+        HP_TRY(run_small_build(L, sk, sa, max_tries, &st));
+        return small_build_outcome(st, seed, max_tries, h_stats);
+    }
     for (uint32_t a = 0; a < max_tries; a++) {
         const uint64_t s = seed + a;
         PeelOut po{};
@@ -1403,6 +1524,20 @@ hpeel_status hpeel_mphf_build_async(const uint64_t *d_keys, uint64_t n, uint64_t
                     lay.total);
     AsyncArgs a{d_keys, (uint32_t)n, (uint32_t)m, max_tries, seed, gamma_milli,
                 d_G, d_rank_dir, d_stats, (char *)d_ws, L.sms};
+    SmallArgs sa{};
+    SmallLaunch sk{};
+    if (max_tries <= kSmallTries &&
+        small_route(1, peel_layout(n, m, 3), n, m, 3, false, (char *)d_ws + lay.peel, &sa, &sk)) {
+        sa.keys = d_keys;
+        sa.fm = make_fastmod(m / 3);
+        sa.seed = seed;
+        sa.max_tries = max_tries;
+        sa.G = d_G;
+        sa.D = d_rank_dir;
+        sa.stats = d_stats;
+        launch_small(L, sk, sa);
+        return check_launch("small build");
+    }
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     HP_CUDA(cudaStreamIsCapturing(L.stream, &cs));
     if (cs == cudaStreamCaptureStatusActive) {
@@ -1474,6 +1609,20 @@ hpeel_status hpeel_sf_build(const uint64_t *d_keys, const uint32_t *d_values, ui
     const uint32_t b = hpeel_sf_bits(sigma);
     const uint64_t words = (m * b + 63) / 64;
     const FastMod fm = make_fastmod(m / 3);
+    SmallArgs sa{};
+    SmallLaunch sk{};
+    if (small_route(2, lay, n, m, 3, false, ws, &sa, &sk)) {
+        sa.keys = d_keys;
+        sa.fm = fm;
+        sa.seed = seed;
+        sa.values = d_values;
+        sa.fs = make_fastmod(sigma);
+        sa.bits = b;
+        sa.U = d_U;
+        hpeel_stats st{};
+        HP_TRY(run_small_build(L, sk, sa, max_tries, &st));
+        return small_build_outcome(st, seed, max_tries, h_stats);
+    }
     for (uint32_t a = 0; a < max_tries; a++) {
         const uint64_t s = seed + a;
         PeelOut po{};
@@ -1549,6 +1698,22 @@ hpeel_status hpeel_sf_build_async(const uint64_t *d_keys, const uint32_t *d_valu
     a.sigma = sigma;
     a.bits = hpeel_sf_bits(sigma);
     a.U = d_U;
+    SmallArgs sa{};
+    SmallLaunch sk{};
+    if (max_tries <= kSmallTries &&
+        small_route(2, peel_layout(n, m, 3), n, m, 3, false, (char *)d_ws + lay.peel, &sa, &sk)) {
+        sa.keys = d_keys;
+        sa.fm = make_fastmod(m / 3);
+        sa.seed = seed;
+        sa.max_tries = max_tries;
+        sa.values = d_values;
+        sa.fs = make_fastmod(sigma);
+        sa.bits = a.bits;
+        sa.U = d_U;
+        sa.stats = d_stats;
+        launch_small(L, sk, sa);
+        return check_launch("small build");
+    }
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     HP_CUDA(cudaStreamIsCapturing(L.stream, &cs));
     if (cs == cudaStreamCaptureStatusActive) {

@@ -307,6 +307,40 @@ void launch_large_rank(const Launch &L, const uint64_t *G, uint64_t m, uint32_t 
 void launch_large_lookup(const Launch &L, const uint64_t *keys, uint64_t nq, FastMod fm,
                          uint64_t seed, const uint64_t *G, const uint64_t *dir, uint64_t *out);
 
+// Small graphs (small.cu): the whole path in one launch of one thread-block
+// cluster.  Inputs and outputs of a launch; small_plan fills in the shape.
+struct SmallArgs {
+    const uint32_t *edges;   // peel: [n][r] rows, or
+    const uint64_t *keys;    // MPHF and static function: keys hashed with (seed, fm)
+    FastMod fm;
+    uint64_t seed;
+    uint32_t max_tries;
+    uint32_t n, m, P;        // P: part size (m for a general graph)
+    uint32_t epc, epc_magic, vslots;  // edges per block, its reciprocal, vertex slots
+    uint32_t max_layers;
+    uint32_t *order, *claim; // or null
+    uint64_t *layer_off;     // or null
+    uint64_t *G, *D;         // MPHF
+    const uint32_t *values;  // static function
+    FastMod fs;
+    uint32_t bits;
+    uint64_t *U;
+    hpeel_stats *stats;      // device memory or pinned host memory
+    unsigned long long *wide;  // workspace: 64-bit vertex records [m]
+};
+struct SmallLaunch {
+    const void *fn;
+    uint32_t blocks, threads;
+    size_t smem;
+};
+// Seeds one launch tries at most.
+constexpr uint32_t kSmallTries = 64;
+// mode 0: peel, 1: MPHF, 2: static function.  False when the graph does not
+// fit a cluster of the current device.
+bool small_plan(int mode, uint64_t n, uint64_t m, uint32_t r, bool gen, SmallArgs *a,
+                SmallLaunch *out);
+void launch_small(const Launch &L, const SmallLaunch &k, const SmallArgs &a);
+
 // a10: batched bucket peel (batched.cu).
 size_t batched_scratch_bytes(uint32_t gamma_milli);
 uint32_t batched_max_gamma_milli();
