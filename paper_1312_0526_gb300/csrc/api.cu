@@ -294,8 +294,8 @@ void destroy_graph(RoundGraph &g) {
 
 // Capture streams of this thread (one per nesting depth of the graph).
 cudaStream_t capture_stream(int depth) {
-    thread_local cudaStream_t s[4] = {nullptr, nullptr, nullptr, nullptr};
-    thread_local int dev_of[4] = {-1, -1, -1, -1};
+    thread_local cudaStream_t s[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+    thread_local int dev_of[5] = {-1, -1, -1, -1, -1};
     int d = 0;
     cudaGetDevice(&d);
     if (!s[depth] || dev_of[depth] != d) {
@@ -377,11 +377,13 @@ hpeel_status launch_cached_graph(const Launch &L, const std::string &key, F capt
 }
 
 // Round 0 and the loops of rounds, added at the capture position of s0; the
-// loop bodies are captured on s1.  With a sorted plan: round 0 and the first
-// rounds in sorted form (a while node over sorted rounds, rounds_bucketed.cu),
-// then a while node over the random round kernel; without one: the random
-// round 0 and its loop.  The round kernels' last blocks (or the sorted
-// rounds' closing kernel) set the loop conditions.
+// loop bodies are captured on s1, a loop inside a loop on s2.  With a sorted
+// plan: round 0 and the first rounds in sorted form (a while node over sorted
+// rounds, rounds_bucketed.cu), then the loop of random rounds; without one: the
+// random round 0 and that loop: a while node whose body is a while node over
+// the round kernel (layers above tail_max), then the cluster kernel that runs
+// small layers until one is empty or large again.  The round kernels' last
+// blocks (or the sorted rounds' closing kernel) set the loop conditions.
 struct RoundsArgs {
     uint32_t n, m, r;
     bool gen;
@@ -393,9 +395,11 @@ struct RoundsArgs {
     uint32_t *loff;
     Ctl *ctl;
     uint32_t max_rounds;
+    TailLaunch tail;
 };
 
-cudaError_t capture_rounds(cudaStream_t s0, cudaStream_t s1, int sms, const RoundsArgs &a) {
+cudaError_t capture_rounds(cudaStream_t s0, cudaStream_t s1, cudaStream_t s2, int sms,
+                           const RoundsArgs &a) {
     Launch L0{s0, sms}, L1{s1, sms};
     const RoundLaunch k0 = round0_launch(L0, a.r, a.gen), k1 = round_launch(L0, a.r, a.gen);
     cudaGraphConditionalHandle h_s = 0, h_r = 0;
@@ -427,19 +431,43 @@ cudaError_t capture_rounds(cudaStream_t s0, cudaStream_t s1, int sms, const Roun
     e = append_conditional(s0, h_r, cudaGraphCondTypeWhile, &body);
     if (e == cudaSuccess) e = begin_body(body);
     if (e != cudaSuccess) return e;
-    {
-        void *args[] = {(void *)&a.prm, &h_r};
-        e = cudaLaunchKernel(k1.fn, dim3(k1.grid), dim3(k1.block), args, k1.smem, s1);
+    // captures end on every path: a stream left capturing would be lost
+    auto end = [](cudaStream_t s, cudaError_t e1) {
+        cudaGraph_t got = nullptr;
+        const cudaError_t e2 = cudaStreamEndCapture(s, &got);
+        return e1 != cudaSuccess ? e1 : e2;
+    };
+    if (a.tail.tail_max == 0) {
+        void *args[] = {(void *)&a.prm, (void *)&a.ctl, &h_r};
+        return end(s1, cudaLaunchKernel(k1.fn, dim3(k1.grid), dim3(k1.block), args, k1.smem, s1));
     }
-    const cudaError_t e2 = cudaStreamEndCapture(s1, &g);
-    return e != cudaSuccess ? e : e2;
+    cudaGraphConditionalHandle h_big = 0;
+    cudaGraph_t inner = nullptr;
+    e = new_handle(s1, 0u, 0u, &h_big);
+    if (e == cudaSuccess) {
+        launch_tail_gate(L1, a.prm, h_big);
+        e = append_conditional(s1, h_big, cudaGraphCondTypeWhile, &inner);
+    }
+    if (e == cudaSuccess)
+        e = cudaStreamBeginCaptureToGraph(s2, inner, nullptr, nullptr, 0,
+                                          cudaStreamCaptureModeRelaxed);
+    if (e == cudaSuccess) {
+        void *args[] = {(void *)&a.prm, (void *)&a.ctl, &h_big};
+        e = end(s2, cudaLaunchKernel(k1.fn, dim3(k1.grid), dim3(k1.block), args, k1.smem, s2));
+    }
+    if (e == cudaSuccess) {
+        void *args[] = {(void *)&a.prm, &h_r};
+        e = launch_cluster(a.tail.fn, a.tail.blocks, a.tail.threads, a.tail.smem, s1, args);
+    }
+    return end(s1, e);
 }
 
 // Kernels one peel's rounds launched, from its control block: round 0 (6 in
-// sorted form), 7 per sorted round, 1 per random round.
+// sorted form), 7 per sorted round, 1 per random round, 2 per run of small
+// layers.
 uint64_t round_kernels(const Ctl &c, bool sorted) {
     const uint64_t rounds = (uint64_t)c.round + (c.more ? 1 : 0);
-    return (sorted ? 6 : 1) + 7ull * c.brounds + (rounds - c.brounds);
+    return (sorted ? 6 : 1) + 7ull * c.brounds + (rounds - c.brounds - c.trounds) + 2ull * c.tails;
 }
 
 // The device-driven round loop of a host-driven peel: round 0 and the loops
@@ -453,12 +481,12 @@ hpeel_status launch_round_graph(const Launch &L, const RoundsArgs &a) {
              (const void *)a.prm, a.n, a.m, a.r, a.gen ? 1 : 0, a.sp ? 1 : 0, tu.bucket_shift,
              tu.bucket_sub_shift, tu.bucket_part_passes, tu.sorted_round_min, L.sms);
     return launch_cached_graph(L, std::string(keybuf), [&](cudaGraph_t *g) -> hpeel_status {
-        cudaStream_t s0 = capture_stream(0), s1 = capture_stream(1);
-        if (!s0 || !s1) return fail(HPEEL_ERR_CUDA, "capture stream creation failed");
+        cudaStream_t s0 = capture_stream(0), s1 = capture_stream(1), s2 = capture_stream(2);
+        if (!s0 || !s1 || !s2) return fail(HPEEL_ERR_CUDA, "capture stream creation failed");
         LaunchCountPause pause;
         cudaError_t e = cudaStreamBeginCapture(s0, cudaStreamCaptureModeRelaxed);
         if (e == cudaSuccess) {
-            e = capture_rounds(s0, s1, L.sms, a);
+            e = capture_rounds(s0, s1, s2, L.sms, a);
             cudaGraph_t got = nullptr;
             const cudaError_t e2 = cudaStreamEndCapture(s0, &got);
             if (e == cudaSuccess) e = e2;
@@ -544,10 +572,12 @@ hpeel_status peel_core_rb(const Launch &L, const PeelIO &io, uint32_t n, uint32_
     hp_prm.m = m;
     hp_prm.P = P;
     hp_prm.max_rounds = lay.max_rounds;
+    const TailLaunch tail = tail_launch(r, io.general);
+    hp_prm.tail_max = tail.tail_max;
     RoundParams *prm = reinterpret_cast<RoundParams *>(ws + lay.params);
     launch_set_params(L, prm, hp_prm);
     RoundsArgs ra{n, m, r, io.general, prm, sorted ? &lay.sp : nullptr, sbufs, st, rec, Ll,
-                  loff, ctl, lay.max_rounds};
+                  loff, ctl, lay.max_rounds, tail};
     auto read_ctl = [&]() -> hpeel_status {
         HP_CUDA(cudaMemcpyAsync(hctl, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, L.stream));
         HP_CUDA(cudaStreamSynchronize(L.stream));
@@ -584,7 +614,7 @@ hpeel_status peel_core_rb(const Launch &L, const PeelIO &io, uint32_t n, uint32_
         while (hctl->more && !hctl->err) {
             {
                 ProfScope ps(L, "rounds");
-                launch_round(L, r, io.general, prm);
+                launch_round(L, r, io.general, prm, ctl);
             }
             HP_TRY(check_launch("round"));
             HP_TRY(read_ctl());
@@ -751,8 +781,8 @@ struct AsyncArgs {
 // capture position), or null to capture a graph of its own into *out.
 hpeel_status capture_async_build(const AsyncArgs &a, cudaStream_t into, cudaGraph_t *out) {
     cudaStream_t s0 = into ? into : capture_stream(0), s1 = capture_stream(1),
-                 s2 = capture_stream(2), s3 = capture_stream(3);
-    if (!s0 || !s1 || !s2 || !s3) return fail(HPEEL_ERR_CUDA, "capture stream creation failed");
+                 s2 = capture_stream(2), s3 = capture_stream(3), s4 = capture_stream(4);
+    if (!s0 || !s1 || !s2 || !s3 || !s4) return fail(HPEEL_ERR_CUDA, "capture stream creation failed");
     LaunchCountPause pause;
     const MphfLayout ml = mphf_layout(a.n, a.gamma_milli);
     char *pw = a.ws + ml.peel;
@@ -778,7 +808,8 @@ hpeel_status capture_async_build(const AsyncArgs &a, cudaStream_t into, cudaGrap
     rp.m = m;
     rp.P = P;
     rp.max_rounds = lay.max_rounds;
-    const RoundLaunch k0 = round0_launch(L0, 3, false), k1 = round_launch(L0, 3, false);
+    const TailLaunch tail = tail_launch(3, false);
+    rp.tail_max = tail.tail_max;
 
     // captures end in this order whatever fails, so no stream of ours stays
     // capturing (the caller's capture is left to the caller)
@@ -858,8 +889,8 @@ hpeel_status capture_async_build(const AsyncArgs &a, cudaStream_t into, cudaGrap
         // round 0, then the loops of rounds (as launch_round_graph)
         RoundsArgs ra{n, m, 3, false, prm, lay.sp.enabled ? &lay.sp : nullptr,
                       lay.sp.enabled ? sorted_bufs(lay, pw) : SortedBufs{}, st, rec, Ll, loff,
-                      ctl, lay.max_rounds};
-        HP_CAP(capture_rounds(s1, s2, a.sms, ra));
+                      ctl, lay.max_rounds, tail};
+        HP_CAP(capture_rounds(s1, s2, s3, a.sms, ra));
         cudaGraph_t g = nullptr;
         if (ra.sp) {
             // a sorted round whose buckets overflowed (a skewed input): the
@@ -875,7 +906,7 @@ hpeel_status capture_async_build(const AsyncArgs &a, cudaStream_t into, cudaGrap
             launch_build_incidence(L2, rec, n, 3, m, st, ctl);
             RoundsArgs rr = ra;
             rr.sp = nullptr;
-            HP_CAP(capture_rounds(s2, s3, a.sms, rr));
+            HP_CAP(capture_rounds(s2, s3, s4, a.sms, rr));
             HP_CAP(cudaStreamEndCapture(s2, &g));
             open = 2;
         }
@@ -947,8 +978,8 @@ struct AsyncPeelArgs {
 
 hpeel_status capture_async_peel(const AsyncPeelArgs &a, cudaStream_t into, cudaGraph_t *out) {
     cudaStream_t s0 = into ? into : capture_stream(0), s1 = capture_stream(1),
-                 s2 = capture_stream(2);
-    if (!s0 || !s1 || !s2) return fail(HPEEL_ERR_CUDA, "capture stream creation failed");
+                 s2 = capture_stream(2), s3 = capture_stream(3);
+    if (!s0 || !s1 || !s2 || !s3) return fail(HPEEL_ERR_CUDA, "capture stream creation failed");
     LaunchCountPause pause;
     const PeelLayout lay = peel_layout(a.n, a.m, a.r, a.general);
     char *ws = a.ws;
@@ -977,7 +1008,8 @@ hpeel_status capture_async_peel(const AsyncPeelArgs &a, cudaStream_t into, cudaG
     rp.m = m;
     rp.P = P;
     rp.max_rounds = lay.max_rounds;
-    const RoundLaunch k0 = round0_launch(L0, r, a.general), k1 = round_launch(L0, r, a.general);
+    const TailLaunch small_tail = tail_launch(r, a.general);
+    rp.tail_max = small_tail.tail_max;
 
     int open = 0;
     const int first = into ? 1 : 0;
@@ -1048,8 +1080,8 @@ hpeel_status capture_async_peel(const AsyncPeelArgs &a, cudaStream_t into, cudaG
     const bool sorted = lay.sp.enabled && !a.general;
     RoundsArgs ra{n, m, r, a.general, prm, sorted ? &lay.sp : nullptr,
                   sorted ? sorted_bufs(lay, ws) : SortedBufs{}, st, rec, Ll, loff, ctl,
-                  lay.max_rounds};
-    HP_CAP(capture_rounds(s0, s1, a.sms, ra));
+                  lay.max_rounds, small_tail};
+    HP_CAP(capture_rounds(s0, s1, s2, a.sms, ra));
     if (sorted) {
         // a sorted round whose buckets overflowed (a skewed input): the build
         // and the rounds are redone in random form
@@ -1064,7 +1096,7 @@ hpeel_status capture_async_peel(const AsyncPeelArgs &a, cudaStream_t into, cudaG
         launch_build_incidence(L1, rec, n, r, m, st, ctl);
         RoundsArgs rr = ra;
         rr.sp = nullptr;
-        HP_CAP(capture_rounds(s1, s2, a.sms, rr));
+        HP_CAP(capture_rounds(s1, s2, s3, a.sms, rr));
         cudaGraph_t g = nullptr;
         HP_CAP(cudaStreamEndCapture(s1, &g));
         open = 1;

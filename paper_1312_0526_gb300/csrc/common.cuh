@@ -23,12 +23,13 @@ enum : uint32_t {
 };
 
 // Device-side control block of one peel (lives in the workspace).
-struct Ctl {
+struct alignas(16) Ctl {
+    uint32_t round;      // index t of the round being run, and the list entries
+    uint32_t lbeg, lend; // [lbeg, lend) of its layer: one 16-byte load
+    uint32_t more;       // 1 while the next layer is non-empty
     uint32_t lcur;       // append cursor of the layer list L (L_0 | L_1 | ...)
-    uint32_t round;      // index t of the round being run
     uint32_t done;       // blocks finished in the current update launch
     uint32_t err;        // first device error code (0 = none)
-    uint32_t more;       // 1 while the next layer is non-empty
     uint32_t next_size;  // size of the layer the next round deletes
     uint32_t cross;      // vertices that fell from degree 2 to 1 (all rounds)
     uint32_t first_layer;   // |L_0|
@@ -37,6 +38,8 @@ struct Ctl {
     uint32_t bmode;      // 1: the next round runs in sorted (bucketed) form
     uint32_t brounds;    // rounds run in sorted form
     uint32_t cvalid;     // 1: the incidence build left round 0's claims in the claim list
+    uint32_t tails;      // launches of the cluster kernel that runs small layers
+    uint32_t trounds;    // rounds it ran
     uint32_t pad[3];
 };
 
@@ -74,6 +77,7 @@ struct RoundParams {
     uint32_t *loff;          // layer starts
     Ctl *ctl;
     uint32_t n, m, P, max_rounds;
+    uint32_t tail_max;       // layers of up to this size run in the cluster kernel (0: none)
 };
 
 // SplitMix64 output function (Steele, Lea, Flood, OOPSLA 2014): two
@@ -318,6 +322,22 @@ __device__ __forceinline__ uint32_t load_entry(const uint4 *L, uint64_t i, uint3
     const uint4 a = __ldcs(L + i);
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = 0u;
     return a.w;
+}
+
+// An entry another SM may just have written (read from L2), and its parts as
+// load_entry gives them.
+template <int R>
+__device__ __forceinline__ Entry<R> load_entry_cg(const uint4 *L, uint64_t i) {
+    Entry<R> x;
+    x.w[0] = __ldcg(L + (R == 4 ? 2 * i : i));
+    if (R == 4) x.w[R == 4 ? 1 : 0] = __ldcg(L + 2 * i + 1);
+    return x;
+}
+template <int R>
+__device__ __forceinline__ uint32_t split_entry(const Entry<R> &x, uint32_t (&v)[4]) {
+    const uint4 a = x.w[0];
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = R == 4 ? a.w : 0u;
+    return R == 4 ? x.w[R == 4 ? 1 : 0].x : a.w;
 }
 
 template <int R>

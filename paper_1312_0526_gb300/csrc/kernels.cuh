@@ -43,6 +43,13 @@ void prof_flush();  // after a stream synchronisation: accumulate timings
 // in between would make that thread's launch fail.
 void smem_optin(const void *fn);
 
+// Largest thread-block cluster (a power of two up to 16; 0: none) the current
+// device runs fn in with these threads and this dynamic shared memory; found
+// once per device and kernel.  launch_cluster: one cluster of `blocks` blocks.
+uint32_t max_cluster(const void *fn, unsigned threads, size_t smem);
+cudaError_t launch_cluster(const void *fn, unsigned blocks, unsigned threads, size_t smem,
+                           cudaStream_t stream, void **args);
+
 // Persistent grid size for grid-stride kernels over device-sized ranges.
 inline unsigned grid_fixed(const Launch &L, int per_sm) { return (unsigned)(L.sms * per_sm); }
 // One wave: as many blocks of kThreads as fit on the device at once (at most
@@ -262,8 +269,19 @@ RoundLaunch round0_launch(const Launch &L, uint32_t r, bool gen);
 
 // a5 + a4 of the next round + a6: delete layer t (t read on the device),
 // claim and list layer t+1, close the round.
-void launch_round(const Launch &L, uint32_t r, bool gen, const RoundParams *prm);
+void launch_round(const Launch &L, uint32_t r, bool gen, const RoundParams *prm, Ctl *ctl);
 RoundLaunch round_launch(const Launch &L, uint32_t r, bool gen);
+
+// Runs of small layers: one cluster peels round after round while the layer
+// holds at most tail_max entries (k_tail); the gate sets h to whether the next
+// layer is larger.
+struct TailLaunch {
+    const void *fn;
+    uint32_t blocks, threads, tail_max;  // tail_max 0: no clusters, no tail
+    size_t smem;
+};
+TailLaunch tail_launch(uint32_t r, bool gen);
+void launch_tail_gate(const Launch &L, const RoundParams *prm, cudaGraphConditionalHandle h);
 
 // claim[e] = claim word of record e.
 void launch_extract_claim(const Launch &L, const uint4 *rec, uint32_t n, uint32_t r,

@@ -49,6 +49,7 @@
 #include <set>
 #include <utility>
 
+#include "cluster.cuh"
 #include "kernels.cuh"
 
 namespace hp {
@@ -162,12 +163,13 @@ void launch_build_incidence(const Launch &L, const uint4 *rec, uint32_t n, uint3
 // may start only after others have finished when the GPU is shared with
 // other work, so the round may advance only once every block has read it.
 // When the launch runs inside a CUDA graph's while node, the last block also
-// sets the node's condition: 1 while the next layer is non-empty, the layer
-// table has room and no kernel has raised an error (the loop ends after at
-// most max_rounds launches whatever happens).
-__device__ __forceinline__ void close_round(Ctl *ctl, uint32_t *loff, uint32_t t,
+// sets the node's condition: 1 while the next layer is non-empty and larger
+// than tail_max (smaller ones go to k_tail), the layer table has room and no
+// kernel has raised an error (the loop ends after at most max_rounds launches
+// whatever happens).
+__device__ __forceinline__ void close_round(Ctl *ctl, uint32_t *loff, uint32_t t, uint32_t beg,
                                             uint32_t crossings, uint32_t moves,
-                                            uint32_t max_rounds,
+                                            uint32_t max_rounds, uint32_t tail_max,
                                             cudaGraphConditionalHandle cond) {
     __shared__ uint32_t s_cnt[2][kThreads / 32];
     const uint32_t wc = __reduce_add_sync(0xFFFFFFFFu, crossings);
@@ -190,20 +192,19 @@ __device__ __forceinline__ void close_round(Ctl *ctl, uint32_t *loff, uint32_t t
         const uint32_t d = atomicAdd(&ctl->done, 1u);
         if (d == gridDim.x - 1) {
             __threadfence();
-            const uint32_t end = atomicAdd(&ctl->lcur, 0u);
-            const uint32_t beg = loff[t + 1];
+            const uint32_t end = __ldcg(&ctl->lcur);
+            const uint32_t err = __ldcg(&ctl->err);
             loff[t + 2] = end;
             uint32_t more = end > beg ? 1u : 0u;
             if (more && t + 2 >= max_rounds) {  // round t+1 would overflow loff
                 more = 0;
                 atomicCAS(&ctl->err, 0u, (uint32_t)kDevCapacity);
             }
-            if (atomicAdd(&ctl->err, 0u) != 0u) more = 0;  // stop on any device error
+            if (err != 0u) more = 0;  // stop on any device error
             ctl->next_size = end - beg;
-            ctl->more = more;
             ctl->done = 0;
-            ctl->round = t + 1;
-            if (cond) cudaGraphSetConditional(cond, more);
+            *reinterpret_cast<uint4 *>(&ctl->round) = make_uint4(t + 1, beg, end, more);
+            if (cond) cudaGraphSetConditional(cond, more && end - beg > tail_max ? 1u : 0u);
         }
     }
 }
@@ -401,9 +402,8 @@ k_round0(const RoundParams *__restrict__ prm, cudaGraphConditionalHandle cond) {
             loff[1] = end;
             ctl->next_size = end;
             ctl->first_layer = end;
-            ctl->more = more;
             ctl->done = 0;
-            ctl->round = 0;
+            *reinterpret_cast<uint4 *>(&ctl->round) = make_uint4(0u, 0u, end, more);
             if (cond) cudaGraphSetConditional(cond, more);
         }
     }
@@ -443,35 +443,33 @@ constexpr int round_u() { return R == 4 ? 2 : HPEEL_ROUND_U; }
 #endif
 template <int R, bool GEN>
 __global__ void __launch_bounds__(kThreads, HPEEL_ROUND_MIN_BLOCKS)
-k_round(const RoundParams *__restrict__ prm, cudaGraphConditionalHandle cond) {
+k_round(const RoundParams *__restrict__ prm, Ctl *__restrict__ ctl,
+        cudaGraphConditionalHandle cond) {
     constexpr int kRoundU = round_u<R>();
     uint4 *__restrict__ Lw = prm->L;
     Entry<R> *__restrict__ Lst = reinterpret_cast<Entry<R> *>(prm->L);
     uint32_t *__restrict__ loff = prm->loff;
     unsigned long long *__restrict__ st = prm->st;
     uint4 *__restrict__ rec = prm->rec;
-    Ctl *ctl = prm->ctl;
     const uint32_t n = prm->n, P = prm->P, max_rounds = prm->max_rounds;
     constexpr int kCap = stage_cap<R, HPEEL_ROUND_STAGE_BYTES>();
     auto stage = warp_stage<R, kCap>();
-    const uint32_t t = *(volatile uint32_t *)&ctl->round;
-    uint32_t lb = loff[t], le = loff[t + 1];
+    const uint4 now = __ldcg(reinterpret_cast<const uint4 *>(&ctl->round));
+    const uint32_t t = now.x;
+    uint32_t lb = now.y, le = now.z;
     if (lb > le || le > n) {  // inconsistent state: report, delete nothing
         raise_err(ctl, kDevCapacity);
         lb = le;
     }
-    constexpr uint32_t kBlockStep = kThreads * kRoundU;
-    // a small layer is spread over as many blocks as it fills; the others
-    // skip the loop but still take part in closing the round
-    const uint64_t need = ((uint64_t)(le - lb) + kBlockStep - 1) / kBlockStep;
-    const uint32_t active = (uint32_t)(need < gridDim.x ? (need ? need : 1) : gridDim.x);
-    const uint64_t stride = (uint64_t)active * kBlockStep;
+    // a small layer is spread over the blocks first (an SM serves one lane's
+    // atomic per cycle), then over their warps; a warp without entries only
+    // takes part in closing the round
+    const uint64_t stride = (uint64_t)gridDim.x * kThreads * kRoundU;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     uint32_t cross = 0, moves = 0;
     const unsigned long long one = 1ull;
-    const uint64_t first = blockIdx.x < active ? lb + (uint64_t)blockIdx.x * kBlockStep +
-                                                     (uint64_t)warp * 32 * kRoundU
-                                               : (uint64_t)le;
+    const uint64_t first =
+        (uint64_t)lb + ((uint64_t)warp * gridDim.x + blockIdx.x) * 32u * kRoundU;
     for (uint64_t base = first; base < le; base += stride) {
         uint32_t e[kRoundU], v[kRoundU][4], hg[kRoundU];
         bool mine[kRoundU];
@@ -516,8 +514,12 @@ k_round(const RoundParams *__restrict__ prm, cudaGraphConditionalHandle cond) {
                 moves++;
             }
         }
-        // vertices that fell to degree 1 mark themselves and claim their last
-        // edge for round t+1; the vertex words of that edge come along
+        // vertices that fell to degree 1 claim their last edge for round t+1,
+        // one (entry, vertex) place of the step after the other; the vertex
+        // words of that edge come along.  Queued per warp and claimed in full
+        // warps instead, more reads that an atomic on the same sector follows
+        // are in flight, and the memory system serves them more slowly: 137
+        // against 124 ms per peel at n = 8e8.
         bool take[kRoundU][R - 1];
         uint32_t f[kRoundU][R - 1], pf[kRoundU][R - 1][4], jf[kRoundU][R - 1];
 #pragma unroll
@@ -563,7 +565,7 @@ k_round(const RoundParams *__restrict__ prm, cudaGraphConditionalHandle cond) {
             }
     }
     stage.flush(&ctl->lcur, Lst);
-    close_round(ctl, loff, t, cross, moves, max_rounds, cond);
+    close_round(ctl, loff, t, le, cross, moves, max_rounds, prm->tail_max, cond);
 }
 
 template <int R>
@@ -575,12 +577,280 @@ RoundLaunch round_launch(const Launch &L, uint32_t r, bool gen) {
         HPEEL_ROUND_STAGE_BYTES);
 }
 
-void launch_round(const Launch &L, uint32_t r, bool gen, const RoundParams *prm) {
+void launch_round(const Launch &L, uint32_t r, bool gen, const RoundParams *prm, Ctl *ctl) {
     const RoundLaunch k = round_launch(L, r, gen);
     cudaGraphConditionalHandle c0 = 0;
-    void *args[] = {(void *)&prm, &c0};
+    void *args[] = {(void *)&prm, (void *)&ctl, &c0};
     count_launch();
     cudaLaunchKernel(k.fn, dim3(k.grid), dim3(k.block), args, k.smem, L.stream);
+}
+
+// ------------------------------------------------------------------ tails --
+// Rounds over small layers, one after the other in one launch of one cluster.
+// A launch of k_round costs 12 us however small its layer is (launch, while
+// node, then eight dependent trips to L2: parameters, round, layer start,
+// entries, atomics, claims, list cursor, closing count), and a peel spends
+// most of its rounds on layers of a few thousand edges; close above the
+// threshold there are hundreds of them.  Here a round is the trips its edges
+// need (entry from shared memory, vertex atomics, claims) and one cluster
+// barrier.  Each block keeps the entries it appends in shared memory: they are
+// its share of the next layer, and when it deletes them it writes them to the
+// layer list, at the place the blocks' counts give it.  When one block has
+// more than kShare entries, the layer goes to the list and is dealt out again.
+// The kernel returns when the layer is empty or larger than tail_max.
+// What bounds a round: an SM serves one lane's atomic per cycle, a trip to L2
+// takes 460 (load) to 890 cycles (64-bit atomic), the barrier 600-800; 4 us
+// per round at 4,000 entries with the graph in L2, 5-7 us from DRAM.  One
+// entry per thread of 1,024 (two per thread of 512: 4,380 instead of 3,460 us
+// for a peel of 1e7 edges at gamma 1.222).  A share of 2,048 entries per block:
+// 1e6-key builds 873 us, 950 with 1,024 (larger layers are as well off with
+// k_round on all SMs).  Peel of 1e7 edges at gamma 1.222 6,090 -> 3,460 us,
+// MPHF build of 1e6 keys 1,440 -> 873 us, of 4e6 1,700 -> 1,360.
+constexpr int kTailThreads = 1024;
+constexpr int kTailU = 1;       // entries per thread in flight
+constexpr int kTailClaims = 2;  // claims per thread in flight
+template <int R>
+constexpr uint32_t tail_cap() { return R == 4 ? 3072u : 4096u; }  // staged entries per block
+template <int R>
+constexpr uint32_t tail_share() { return R == 4 ? 1024u : 2048u; }  // entries a block may delete
+
+template <int R, bool GEN>
+__global__ void __launch_bounds__(kTailThreads, 1)
+k_tail(const RoundParams *__restrict__ prm, cudaGraphConditionalHandle cond) {
+    constexpr uint32_t kCap = tail_cap<R>(), kShare = tail_share<R>();
+    static_assert(kShare * (R - 1) <= kCap, "a block's share of a layer cannot overflow its stage");
+    extern __shared__ uint4 dyn_smem[];
+    __shared__ uint32_t s_cnt[2], s_slot[2][16];
+    __shared__ uint2 s_queue[kTailThreads / 32][32 * kTailU * (R - 1)];
+    Entry<R> *const stage = reinterpret_cast<Entry<R> *>(dyn_smem);  // [2][kCap]
+    uint4 *const Lw = prm->L;
+    uint32_t *const loff = prm->loff;
+    unsigned long long *const st = prm->st;
+    uint4 *const rec = prm->rec;
+    Ctl *const ctl = prm->ctl;
+    const uint32_t n = prm->n, P = prm->P, max_rounds = prm->max_rounds, tail_max = prm->tail_max;
+    const uint32_t rank = cl_rank(), blocks = gridDim.x;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    uint2 *const queue = s_queue[warp];
+    const uint4 now = __ldcg(reinterpret_cast<const uint4 *>(&ctl->round));
+    uint32_t more = __ldcg(&ctl->err) ? 0u : now.w;
+    const uint32_t t0 = now.x;
+    uint32_t t = t0, lb = now.y, le = now.z;
+    // nothing to do, or a state the loop around cannot leave behind: stop it
+    // (the same decision in every block)
+    const bool bad = more && (lb >= le || le > n || le - lb > tail_max);
+    if (!more || bad) {
+        if (rank == 0 && tid == 0) {
+            if (bad) {
+                raise_err(ctl, kDevCapacity);
+                ctl->more = 0;
+            }
+            if (cond) cudaGraphSetConditional(cond, 0u);
+        }
+        return;
+    }
+    if (tid < 2) s_cnt[tid] = 0;
+    cl_sync<false>();
+    // this block's entries: c of them, at list position p0; staged in buffer
+    // b, or read from the list
+    bool staged = false;
+    uint32_t b = 0, per = (le - lb + blocks - 1) / blocks;
+    uint32_t p0 = min(lb + rank * per, le), c = min(per, le - p0);
+    uint32_t cross = 0, moves = 0;
+    for (;;) {
+        const uint32_t nb = b ^ 1u;
+        Entry<R> *const next = stage + nb * kCap;
+        for (uint32_t base = warp * 32u * kTailU; base < c; base += kTailThreads * kTailU) {
+            uint32_t e[kTailU], v[kTailU][4], hg[kTailU];
+            bool mine[kTailU];
+#pragma unroll
+            for (int u = 0; u < kTailU; u++) {
+                const uint32_t i = base + (uint32_t)u * 32u + lane;
+                mine[u] = i < c;
+                e[u] = hg[u] = 0;
+#pragma unroll
+                for (int k = 0; k < 4; k++) v[u][k] = 0;
+                if (mine[u]) {
+                    const Entry<R> x = staged ? stage[b * kCap + i] : load_entry_cg<R>(Lw, p0 + i);
+                    const uint32_t w = split_entry<R>(x, v[u]);
+                    e[u] = GEN ? w & kGenIdMask : w;
+                    hg[u] = GEN ? w >> kGenPosShift : part_of<R>(v[u][0], P);
+                }
+            }
+            unsigned long long old[kTailU][R - 1];
+#pragma unroll
+            for (int u = 0; u < kTailU; u++) {
+                const unsigned long long sub = 0ull - (((unsigned long long)e[u] << 32) | 1ull);
+#pragma unroll
+                for (int k = 0; k < R - 1; k++)
+                    old[u][k] = mine[u] ? atomicAdd(st + v[u][k + 1], sub) : 0ull;
+            }
+            // the entry, with its hinge corrected (as in k_round)
+#pragma unroll
+            for (int u = 0; u < kTailU; u++) {
+                uint32_t h = hg[u];
+#pragma unroll
+                for (int k = R - 2; k >= 0; k--) {
+                    const uint32_t pos = (uint32_t)k + ((uint32_t)k >= hg[u] ? 1u : 0u);
+                    if (((uint32_t)old[u][k] & kMark) && pos < h) h = pos;
+                }
+                if (mine[u] && (staged || h != hg[u])) {
+                    uint32_t p[4], q[4];
+                    unrotate<R>(v[u], hg[u], p);
+                    rotate_to<R>(p, h, q);
+                    store_entry<R>(Lw, p0 + base + (uint32_t)u * 32u + lane,
+                                   make_entry<R>(q, entry_id<GEN>(e[u], h)));
+                    if (h != hg[u]) moves++;
+                }
+            }
+            // the vertices that fell to degree 1 are queued {vertex, edge} and
+            // claim in full warps: their requests go out together
+            uint32_t qn = 0;
+#pragma unroll
+            for (int u = 0; u < kTailU; u++)
+#pragma unroll
+                for (int k = 0; k < R - 1; k++) {
+                    bool one = mine[u] && (uint32_t)old[u][k] == 2u;
+                    const uint32_t f = (uint32_t)(old[u][k] >> 32) - e[u];
+                    cross += one ? 1u : 0u;
+                    if (one && f >= n) {
+                        raise_err(ctl, kDevBadEdge);
+                        one = false;
+                    }
+                    const uint32_t who = __ballot_sync(0xFFFFFFFFu, one);
+                    if (one) queue[qn + __popc(who & ((1u << lane) - 1u))] = make_uint2(v[u][k + 1], f);
+                    qn += __popc(who);
+                }
+            __syncwarp();
+            for (uint32_t q0 = 0; q0 < qn; q0 += 32u * kTailClaims) {
+                uint2 it[kTailClaims];
+                bool on[kTailClaims];
+                uint32_t pf[kTailClaims][4], jf[kTailClaims], cw[kTailClaims];
+#pragma unroll
+                for (int d = 0; d < kTailClaims; d++) {
+                    const uint32_t k = q0 + (uint32_t)d * 32u + lane;
+                    on[d] = k < qn;
+                    it[d] = on[d] ? queue[k] : make_uint2(0u, 0u);
+                    jf[d] = cw[d] = 0;
+#pragma unroll
+                    for (int q = 0; q < 4; q++) pf[d][q] = 0;
+                    if (!on[d]) continue;
+                    if (GEN) {
+                        cw[d] = claim_and_read<R, GEN>(rec, it[d].y, (t + 1) << 2, it[d].x, P, pf[d],
+                                                       jf[d]);
+                    } else {
+                        // record and claim word side by side: an r-partite
+                        // position needs no row, and few requests are in
+                        // flight here (see claim_and_read for many)
+                        jf[d] = part_of<R>(it[d].x, P);
+                        const uint4 q =
+                            __ldcg(rec + (R == 4 ? 2 * (uint64_t)it[d].y : (uint64_t)it[d].y));
+                        cw[d] = atomicMin(claim_ptr<R>(rec, it[d].y), ((t + 1) << 2) | jf[d]);
+                        pf[d][0] = q.x;
+                        pf[d][1] = q.y;
+                        pf[d][2] = R >= 3 ? q.z : 0u;
+                        pf[d][3] = R == 4 ? q.w : 0u;
+                    }
+                }
+                // first claimers append their entry, others mark a lowered claim
+                uint32_t at[kTailClaims], total = 0;
+#pragma unroll
+                for (int d = 0; d < kTailClaims; d++) {
+                    const bool take = on[d] && cw[d] == kUnclaimed;
+                    if (on[d] && !take && (((t + 1) << 2) | jf[d]) < cw[d])
+                        atomicOr(reinterpret_cast<unsigned int *>(st + it[d].x), kMark);
+                    const uint32_t who = __ballot_sync(0xFFFFFFFFu, take);
+                    at[d] = take ? total + __popc(who & ((1u << lane) - 1u)) : 0xFFFFFFFFu;
+                    total += __popc(who);
+                }
+                uint32_t at0 = 0;
+                if (lane == 0 && total) at0 = atomicAdd(&s_cnt[nb], total);
+                at0 = __shfl_sync(0xFFFFFFFFu, at0, 0);
+#pragma unroll
+                for (int d = 0; d < kTailClaims; d++)
+                    if (at[d] != 0xFFFFFFFFu) {
+                        uint32_t q[4];
+                        rotate_to<R>(pf[d], jf[d], q);
+                        next[at0 + at[d]] = make_entry<R>(q, entry_id<GEN>(it[d].y, jf[d]));
+                    }
+            }
+            __syncwarp();  // the queue is filled again
+        }
+        __syncthreads();
+        // every block's count to every block
+        const uint32_t own = *(volatile uint32_t *)&s_cnt[nb];
+        if (tid < blocks) cl_store<false>(cl_map<false>(smem_u32(&s_slot[nb][rank]), tid), own);
+        if (tid == 0) s_cnt[b] = 0;  // appended to from the next round on
+        cl_sync<false>();
+        const uint32_t cl = lane < blocks ? *(volatile uint32_t *)&s_slot[nb][lane] : 0u;
+        const uint32_t size = __reduce_add_sync(0xFFFFFFFFu, cl);
+        const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, lane < rank ? cl : 0u);
+        const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, cl);
+        t++;
+        lb = le;
+        le = lb + size;
+        if (rank == 0 && tid == 0) loff[t + 1] = le;
+        p0 = lb + before;
+        c = own;
+        b = nb;
+        staged = true;
+        if (size == 0) {
+            more = 0;
+            break;
+        }
+        if (t + 1 >= max_rounds) {  // the next round would overflow loff
+            if (rank == 0 && tid == 0) raise_err(ctl, kDevCapacity);
+            more = 0;
+            break;
+        }
+        if (size > tail_max || most > kShare) {
+            for (uint32_t i = tid; i < c; i += kTailThreads)
+                store_entry<R>(Lw, p0 + i, stage[b * kCap + i]);
+            if (size > tail_max) break;
+            cl_sync<false>();
+            staged = false;
+            per = (size + blocks - 1) / blocks;
+            p0 = min(lb + rank * per, le);
+            c = min(per, le - p0);
+        }
+    }
+    cross = __reduce_add_sync(0xFFFFFFFFu, cross);
+    moves = __reduce_add_sync(0xFFFFFFFFu, moves);
+    if (lane == 0 && cross) atomicAdd(&ctl->cross, cross);
+    if (lane == 0 && moves) atomicAdd(&ctl->moves, moves);
+    if (rank == 0 && tid == 0) {
+        if (atomicAdd(&ctl->err, 0u) != 0u) more = 0;
+        *reinterpret_cast<uint4 *>(&ctl->round) = make_uint4(t, lb, le, more);
+        ctl->lcur = le;
+        ctl->next_size = le - lb;
+        ctl->tails++;
+        ctl->trounds += t - t0;
+        if (cond) cudaGraphSetConditional(cond, more);
+    }
+}
+
+// h = the next layer is too large for k_tail.
+__global__ void k_tail_gate(const RoundParams *prm, cudaGraphConditionalHandle h) {
+    const Ctl *ctl = prm->ctl;
+    cudaGraphSetConditional(
+        h, ctl->more && ctl->err == 0u && ctl->next_size > prm->tail_max ? 1u : 0u);
+}
+
+void launch_tail_gate(const Launch &L, const RoundParams *prm, cudaGraphConditionalHandle h) {
+    count_launch();
+    k_tail_gate<<<1, 1, 0, L.stream>>>(prm, h);
+}
+
+TailLaunch tail_launch(uint32_t r, bool gen) {
+    TailLaunch k{};
+    k.fn = r == 2 ? (gen ? (const void *)k_tail<2, true> : (const void *)k_tail<2, false>)
+                  : (r == 3 ? (gen ? (const void *)k_tail<3, true> : (const void *)k_tail<3, false>)
+                            : (gen ? (const void *)k_tail<4, true> : (const void *)k_tail<4, false>));
+    k.threads = kTailThreads;
+    k.smem = r == 4 ? 2 * tail_cap<4>() * sizeof(Entry<4>) : 2 * tail_cap<3>() * sizeof(Entry<3>);
+    k.blocks = max_cluster(k.fn, k.threads, k.smem);
+    if (k.blocks >= 8) k.tail_max = k.blocks * (r == 4 ? tail_share<4>() : tail_share<3>());
+    return k;
 }
 
 // --------------------------------------------------------------- claims --

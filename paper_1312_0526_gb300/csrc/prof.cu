@@ -79,6 +79,59 @@ void smem_optin(const void *fn) {
     cudaGetLastError();
 }
 
+uint32_t max_cluster(const void *fn, unsigned threads, size_t smem) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void *>, uint32_t> known;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    std::lock_guard<std::mutex> lk(mu);
+    const auto it = known.find({dev, fn});
+    if (it != known.end()) return it->second;
+    smem_optin(fn);
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+        cudaGetLastError();
+    uint32_t best = 0;
+    for (uint32_t b = 1; b <= 16; b *= 2) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(b);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = b;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) != cudaSuccess)
+            cudaGetLastError();
+        else if (clusters > 0)
+            best = b;
+    }
+    known[{dev, fn}] = best;
+    return best;
+}
+
+cudaError_t launch_cluster(const void *fn, unsigned blocks, unsigned threads, size_t smem,
+                           cudaStream_t stream, void **args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = blocks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = blocks > 1 ? 1 : 0;
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
+
 void count_launch(uint32_t kernels) {
     if (t_count_pause == 0) g_launches.fetch_add(kernels, std::memory_order_relaxed);
 }

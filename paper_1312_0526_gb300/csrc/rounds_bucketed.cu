@@ -649,8 +649,10 @@ __global__ void k_sorted_close(Ctl *ctl, uint32_t *loff, uint32_t max_rounds, ui
         ctl->first_layer = end;
         next = end;
         more = end > 0 ? 1u : 0u;
+        ctl->lbeg = 0;
     } else {
         const uint32_t beg = loff[t + 1];
+        ctl->lbeg = beg;
         loff[t + 2] = end;
         next = end - beg;
         more = end > beg ? 1u : 0u;
@@ -663,6 +665,7 @@ __global__ void k_sorted_close(Ctl *ctl, uint32_t *loff, uint32_t max_rounds, ui
     }
     if (err) more = 0;  // stop on any device error
     const uint32_t sorted = more && next >= min_edges && next <= max_edges ? 1u : 0u;
+    ctl->lend = end;
     ctl->next_size = next;
     ctl->more = more;
     ctl->bmode = sorted;

@@ -41,10 +41,7 @@
 //               shows two rounds late: one warp per block gathers the blocks'
 //               "deleted something" flags of round t during round t + 1, and
 //               everyone reads the outcome in round t + 2.
-#include <map>
-#include <mutex>
-#include <utility>
-
+#include "cluster.cuh"
 #include "kernels.cuh"
 
 namespace hp {
@@ -62,83 +59,6 @@ constexpr uint32_t kSmBins = 256;                  // layers per pass of the ord
 constexpr uint32_t kSmWarpGroups = 16;             // groups of 32 edges per warp at most
 constexpr uint32_t kSmGroup = 9;                   // log2 of the vertices per group
 constexpr size_t kSmMaxSmem = 224u << 10;          // dynamic shared memory of a block
-
-// ------------------------------------------------- cluster shared memory --
-// SOLO: a cluster of one block, whose accesses are plain shared-memory ones.
-__device__ __forceinline__ uint32_t cl_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-template <bool SOLO>
-__device__ __forceinline__ void cl_sync() {
-    if (SOLO) {
-        __syncthreads();
-    } else {
-        __syncwarp();
-        asm volatile("barrier.cluster.arrive.release.aligned;\n"
-                     "barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    }
-}
-// address of this block's shared address a in block `rank`
-template <bool SOLO>
-__device__ __forceinline__ uint32_t cl_map(uint32_t a, uint32_t rank) {
-    if (SOLO) return a;
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
-template <bool SOLO>
-__device__ __forceinline__ uint32_t cl_load(uint32_t a) {
-    uint32_t v;
-    if (SOLO)
-        asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-    else
-        asm volatile("ld.relaxed.cluster.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-    return v;
-}
-template <bool SOLO>
-__device__ __forceinline__ void cl_store(uint32_t a, uint32_t v) {
-    if (SOLO)
-        asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-    else
-        asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-template <bool SOLO>
-__device__ __forceinline__ uint32_t cl_add(uint32_t a, uint32_t v) {
-    uint32_t old;
-    if (SOLO)
-        asm volatile("atom.relaxed.cta.shared::cta.add.u32 %0, [%1], %2;"
-                     : "=r"(old) : "r"(a), "r"(v) : "memory");
-    else
-        asm volatile("atom.relaxed.cluster.shared::cluster.add.u32 %0, [%1], %2;"
-                     : "=r"(old) : "r"(a), "r"(v) : "memory");
-    return old;
-}
-template <bool SOLO>
-__device__ __forceinline__ void cl_red_add(uint32_t a, uint32_t v) {
-    if (SOLO)
-        asm volatile("red.relaxed.cta.shared::cta.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-    else
-        asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(a), "r"(v)
-                     : "memory");
-}
-template <bool SOLO>
-__device__ __forceinline__ void cl_red_or(uint32_t a, uint32_t v) {
-    if (SOLO)
-        asm volatile("red.relaxed.cta.shared::cta.or.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-    else
-        asm volatile("red.relaxed.cluster.shared::cluster.or.b32 [%0], %1;" ::"r"(a), "r"(v)
-                     : "memory");
-}
-template <bool SOLO>
-__device__ __forceinline__ void cl_red_min(uint32_t a, uint32_t v) {
-    if (SOLO)
-        asm volatile("red.relaxed.cta.shared::cta.min.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-    else
-        asm volatile("red.relaxed.cluster.shared::cluster.min.u32 [%0], %1;" ::"r"(a), "r"(v)
-                     : "memory");
-}
 
 // ------------------------------------------------------------ one block --
 struct SmallShared {
@@ -913,54 +833,6 @@ bool shape_ok(const SmallShape &s) {
     return s.smem <= kSmMaxSmem && s.epc <= s.ept * (s.threads - (s.blocks > 1 ? 32u : 0u));
 }
 
-// Largest cluster of `blocks` the device can run with this kernel and smem.
-bool cluster_fits(const void *fn, const SmallShape &s) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(s.blocks);
-    cfg.blockDim = dim3(s.threads);
-    cfg.dynamicSmemBytes = s.smem;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = s.blocks;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return clusters > 0;
-}
-
-// Largest cluster size of the current device for the largest shared-memory
-// request (0: none), found once per device and kernel.
-uint32_t max_cluster(const void *fn) {
-    static std::mutex mu;
-    static std::map<std::pair<int, const void *>, uint32_t> known;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    std::lock_guard<std::mutex> lk(mu);
-    const auto it = known.find({dev, fn});
-    if (it != known.end()) return it->second;
-    smem_optin(fn);
-    uint32_t best = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-        cudaGetLastError();
-    for (uint32_t b = 1; b <= 16; b *= 2) {
-        SmallShape s{};
-        s.blocks = b;
-        s.threads = kSmThreads;
-        s.smem = kSmMaxSmem;
-        if (cluster_fits(fn, s)) best = b;
-    }
-    known[{dev, fn}] = best;
-    return best;
-}
-
 }  // namespace
 
 bool small_plan(int mode, uint64_t n, uint64_t m, uint32_t r, bool gen, SmallArgs *a,
@@ -976,7 +848,7 @@ bool small_plan(int mode, uint64_t n, uint64_t m, uint32_t r, bool gen, SmallArg
         smem_optin(fn);
     } else {
         fn = small_fn(mode, r, gen, false, 16);
-        const uint32_t most = max_cluster(fn);
+        const uint32_t most = max_cluster(fn, kSmThreads, kSmMaxSmem);
         if (most < 2) return false;
         s = small_shape((uint32_t)n, (uint32_t)m, r, gen, most);
         if (!shape_ok(s)) return false;
@@ -995,20 +867,9 @@ bool small_plan(int mode, uint64_t n, uint64_t m, uint32_t r, bool gen, SmallArg
 }
 
 void launch_small(const Launch &L, const SmallLaunch &k, const SmallArgs &a) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(k.blocks);
-    cfg.blockDim = dim3(k.threads);
-    cfg.dynamicSmemBytes = k.smem;
-    cfg.stream = L.stream;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = k.blocks;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = k.blocks > 1 ? 1 : 0;
     void *args[] = {(void *)&a};
     count_launch();
-    cudaLaunchKernelExC(&cfg, k.fn, args);
+    launch_cluster(k.fn, k.blocks, k.threads, k.smem, L.stream, args);
 }
 
 }  // namespace hp
