@@ -184,6 +184,18 @@ hpeel_stats *pinned_stats() {
     return p;
 }
 
+// The layer starts of a host-decided peel, read back with its control block
+// for the assignment: the first kHeadLayers + 1 of them (a peel with more
+// rounds reads its table in a second copy).
+constexpr uint32_t kHeadLayers = 1023;
+uint32_t *pinned_loff() {
+    thread_local uint32_t *p = nullptr;
+    if (!p) {
+        if (cudaMallocHost((void **)&p, 4 * (kHeadLayers + 1)) != cudaSuccess) p = nullptr;
+    }
+    return p;
+}
+
 struct PeelOut {
     uint32_t rounds;
     uint64_t n_peeled;
@@ -192,6 +204,7 @@ struct PeelOut {
     uint64_t moves;
     uint32_t sorted_rounds;
     uint32_t *loff;  // device layer table (uint32[rounds + 2])
+    const uint32_t *loff_h;  // its first rounds + 1 entries (PeelIO::loff_h), or null
     uint4 *list;     // device layer list: entries {v_hinge, others, e}
 };
 
@@ -207,6 +220,7 @@ struct PeelIO {
     bool general = false;       // a general (not r-partite) hypergraph on [0, m)
     bool host_loop = false;     // launch every round from the host, whatever the tuning
     bool random_rounds = false; // no round in sorted form
+    std::vector<uint32_t> *loff_h = nullptr;  // read the layer starts back (space for long ones)
 };
 
 // Graphs that fit the shared memory of one thread-block cluster are peeled
@@ -624,6 +638,13 @@ hpeel_status peel_core_rb(const Launch &L, const PeelIO &io, uint32_t n, uint32_
         // back to back on the device, one read-back at the end
         ProfScope ps(L, "rounds");
         HP_TRY(launch_round_graph(L, ra));
+        if (io.loff_h) {
+            uint32_t *head = pinned_loff();
+            if (!head) return fail(HPEEL_ERR_CUDA, "cudaMallocHost of the layer starts failed");
+            HP_CUDA(cudaMemcpyAsync(head, loff,
+                                    4 * (size_t)std::min(kHeadLayers, lay.max_rounds + 1) + 4,
+                                    cudaMemcpyDeviceToHost, L.stream));
+        }
         HP_TRY(read_ctl());
         count_launch((uint32_t)round_kernels(*hctl, sorted));
     }
@@ -656,6 +677,17 @@ hpeel_status peel_core_rb(const Launch &L, const PeelIO &io, uint32_t n, uint32_
     out->sorted_rounds = hctl->brounds;
     out->loff = loff;
     out->list = Ll;
+    if (io.loff_h) {
+        if (R <= kHeadLayers && !(tu.host_round_loop || io.host_loop)) {
+            out->loff_h = pinned_loff();
+        } else {
+            io.loff_h->resize((size_t)R + 1);
+            HP_CUDA(cudaMemcpyAsync(io.loff_h->data(), loff, 4 * ((size_t)R + 1),
+                                    cudaMemcpyDeviceToHost, L.stream));
+            HP_CUDA(cudaStreamSynchronize(L.stream));
+            out->loff_h = io.loff_h->data();
+        }
+    }
 
     if (!io.order && !io.claim) return HPEEL_OK;
     if (!io.order) {
@@ -930,12 +962,9 @@ hpeel_status capture_async_build(const AsyncArgs &a, cudaStream_t into, cudaGrap
         HP_CAP(append_conditional(s1, h_asg, cudaGraphCondTypeWhile, &b_asg));
         HP_CAP(begin_body(s2, b_asg));
         open = 3;
-        if (a.values)
-            launch_sf_assign_layer_at(L2, Ll, loff, &state->t, a.values, a.sigma, a.bits, a.U,
-                                      ctl);
-        else
-            launch_assign_layer_at(L2, Ll, loff, &state->t, P, a.G);
-        launch_async_assign_step(L2, state, h_asg);
+        const AssignArgs as{Ll, loff, P, a.values ? a.U : a.G, a.values, make_fastmod(a.sigma),
+                            a.bits, ctl};
+        launch_assign_body(L2, a.values != nullptr, as, state, h_asg);
         cudaGraph_t g = nullptr;
         HP_CAP(cudaStreamEndCapture(s2, &g));
         open = 2;
@@ -1472,6 +1501,7 @@ hpeel_status hpeel_mphf_build(const uint64_t *d_keys, uint64_t n, uint64_t seed,
         HP_TRY(run_small_build(L, sk, sa, max_tries, &st));
         return small_build_outcome(st, seed, max_tries, h_stats);
     }
+    std::vector<uint32_t> loff_h;
     for (uint32_t a = 0; a < max_tries; a++) {
         const uint64_t s = seed + a;
         PeelOut po{};
@@ -1480,6 +1510,7 @@ hpeel_status hpeel_mphf_build(const uint64_t *d_keys, uint64_t n, uint64_t seed,
         io.seed = s;
         io.fm = fm;
         io.order = d_order;
+        io.loff_h = &loff_h;
         HP_TRY(peel_core(L, io, (uint32_t)n, (uint32_t)m, 3, ws + lay.peel, &po));
         if (h_stats) {
             h_stats->attempts = a + 1;
@@ -1503,9 +1534,11 @@ hpeel_status hpeel_mphf_build(const uint64_t *d_keys, uint64_t n, uint64_t seed,
         // a8: reverse layer order
         const uint64_t words = (m + 31) / 32;
         HP_CUDA(cudaMemsetAsync(d_G, 0, 8 * words, L2.stream));
-        for (int64_t t = (int64_t)po.rounds - 1; t >= 0; t--) {
+        {
             ProfScope ps(L2, "assign");
-            launch_assign_layer(L2, po.list, po.loff, (uint32_t)t, (uint32_t)(m / 3), d_G);
+            const AssignArgs as{po.list, po.loff, (uint32_t)(m / 3), d_G, nullptr, FastMod{0, 0}, 0,
+                                nullptr};
+            launch_assign(L2, false, as, po.loff_h, po.rounds);
         }
         HP_TRY(check_launch("assign"));
         // a9: rank directory
@@ -1655,6 +1688,7 @@ hpeel_status hpeel_sf_build(const uint64_t *d_keys, const uint32_t *d_values, ui
         HP_TRY(run_small_build(L, sk, sa, max_tries, &st));
         return small_build_outcome(st, seed, max_tries, h_stats);
     }
+    std::vector<uint32_t> loff_h;
     for (uint32_t a = 0; a < max_tries; a++) {
         const uint64_t s = seed + a;
         PeelOut po{};
@@ -1662,6 +1696,7 @@ hpeel_status hpeel_sf_build(const uint64_t *d_keys, const uint32_t *d_values, ui
         io.keys = d_keys;
         io.seed = s;
         io.fm = fm;
+        io.loff_h = &loff_h;
         HP_TRY(peel_core(L, io, (uint32_t)n, (uint32_t)m, 3, ws, &po));
         if (h_stats) {
             h_stats->attempts = a + 1;
@@ -1676,9 +1711,11 @@ hpeel_status hpeel_sf_build(const uint64_t *d_keys, const uint32_t *d_values, ui
         if (po.n_peeled < n) continue;
         // reverse layer order (sec. 3, sec. 4.3 "Avoiding backward scans")
         HP_CUDA(cudaMemsetAsync(d_U, 0, 8 * words, L.stream));
-        for (int64_t t = (int64_t)po.rounds - 1; t >= 0; t--) {
+        {
             ProfScope ps(L, "sf_assign");
-            launch_sf_assign_layer(L, po.list, po.loff, (uint32_t)t, d_values, sigma, b, d_U, ctl);
+            const AssignArgs as{po.list, po.loff, (uint32_t)(m / 3), d_U, d_values,
+                                make_fastmod(sigma), b, ctl};
+            launch_assign(L, true, as, po.loff_h, po.rounds);
         }
         HP_TRY(check_launch("sf_assign"));
         uint32_t err = 0;

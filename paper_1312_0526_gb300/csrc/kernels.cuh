@@ -378,25 +378,29 @@ size_t scan_tmp_words(uint64_t count);
 void launch_scan_u32(const Launch &L, const uint32_t *in, uint32_t *out, uint64_t count,
                      uint32_t *tmp);
 
-// a8: MWHC assignment of one layer t from its solve records (host loop runs
-// t = R-1 .. 0).
-void launch_assign_layer(const Launch &L, const uint4 *Lst, const uint32_t *loff, uint32_t t,
-                         uint32_t P, uint64_t *G);
-// Static function (sec. 3): assignment of layer t mod sigma, b-bit values;
-// lookup of nq keys.
-void launch_sf_assign_layer(const Launch &L, const uint4 *Lst, const uint32_t *loff, uint32_t t,
-                            const uint32_t *values, uint64_t sigma, uint32_t b, uint64_t *U,
-                            Ctl *ctl);
-void launch_sf_assign_layer_at(const Launch &L, const uint4 *Lst, const uint32_t *loff,
-                               const int32_t *t, const uint32_t *values, uint64_t sigma,
-                               uint32_t b, uint64_t *U, Ctl *ctl);
+// a8: MWHC assignment from the solve records, or that of a static function
+// (sec. 3: mod sigma, b-bit values of the bit string G; values[e] the value of
+// key e).
+struct AssignArgs {
+    const uint4 *Lst;
+    const uint32_t *loff;
+    uint32_t P;
+    uint64_t *G;
+    const uint32_t *values;  // static function
+    FastMod fs;
+    uint32_t b;
+    Ctl *ctl;
+};
+// All layers, last to first, their starts in host memory.
+void launch_assign(const Launch &L, bool sf, const AssignArgs &a, const uint32_t *loff_h,
+                   uint32_t rounds);
+// Body of the device-driven loop over layers (s->t: the next one): solves at
+// least one layer and sets h.
+void launch_assign_body(const Launch &L, bool sf, const AssignArgs &a, AsyncState *s,
+                        cudaGraphConditionalHandle h);
 void launch_sf_lookup(const Launch &L, const uint64_t *keys, uint64_t nq, FastMod fm,
                       uint64_t seed, uint64_t sigma, uint32_t b, const uint64_t *U,
                       uint32_t *out);
-// Assignment of the layer whose index the device holds at *t (device-driven
-// build).
-void launch_assign_layer_at(const Launch &L, const uint4 *Lst, const uint32_t *loff,
-                            const int32_t *t, uint32_t P, uint64_t *G);
 // Device-driven build control (async.cu): one-thread kernels that set the
 // conditions of the graph's loops.
 void launch_async_empty(const Launch &L, hpeel_stats *out, uint64_t seed, uint64_t *D);

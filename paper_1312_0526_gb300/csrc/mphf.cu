@@ -11,76 +11,256 @@
 // their bits with atomicOr.
 // sec. 5: the rank counts non-zero 2-bit pairs of a word with a broadword
 // expression instead of a bit loop.
+#include "cluster.cuh"
 #include "kernels.cuh"
 
 namespace hp {
 
-// Solve the list entries [lb, le) of one layer: each {v_hinge, v_a, v_b, e}
-// with the hinge position the part of v_hinge, read as a stream.  A thread
-// takes kAssignU entries at a time and issues all their loads first.
-#ifndef HPEEL_ASSIGN_U
-#define HPEEL_ASSIGN_U 4
-#endif
-constexpr int kAssignU = HPEEL_ASSIGN_U;
+// ------------------------------------------------------ static functions --
+// sec. 3: any f: S -> [sigma] is stored as u with f(x) = u[h0] + u[h1] +
+// u[h2] mod sigma, b = ceil(log2 sigma) bits per vertex in one bit string
+// (vertex v at bits [v b, (v + 1) b), bit i in word i / 64): a value may
+// straddle two words, so it is read from one or two words and set with one
+// or two atomicOr.  The MPHF is the case sigma = 3, f = hinge.
+__device__ __forceinline__ uint64_t u_get(const uint64_t *U, uint32_t v, uint32_t b) {
+    const uint64_t bit = (uint64_t)v * b;
+    const uint64_t w = bit >> 6;
+    const uint32_t sh = (uint32_t)(bit & 63u);
+    uint64_t x = __ldcg(U + w) >> sh;
+    if (sh + b > 64) x |= __ldcg(U + w + 1) << (64 - sh);
+    return x & ((1ull << b) - 1ull);  // b <= 32
+}
 
-__device__ __forceinline__ void assign_range(const uint4 *__restrict__ Lst, uint32_t lb,
-                                             uint32_t le, uint32_t P, uint64_t *G) {
-    const uint64_t stride = (uint64_t)gridDim.x * kThreads * kAssignU;
-    for (uint64_t i0 = lb + (uint64_t)blockIdx.x * kThreads * kAssignU + threadIdx.x; i0 < le;
-         i0 += stride) {
-        uint4 s[kAssignU];
-#pragma unroll
-        for (int u = 0; u < kAssignU; u++) {
-            const uint64_t i = i0 + (uint64_t)u * kThreads;
-            s[u] = i < le ? __ldcs(Lst + i) : make_uint4(0u, 0u, 0u, 0u);
+__device__ __forceinline__ void u_or(uint64_t *U, uint32_t v, uint32_t b, uint64_t x) {
+    const uint64_t bit = (uint64_t)v * b;
+    const uint64_t w = bit >> 6;
+    const uint32_t sh = (uint32_t)(bit & 63u);
+    atomicOr((unsigned long long *)(U + w), (unsigned long long)(x << sh));
+    if (sh + b > 64) atomicOr((unsigned long long *)(U + w + 1), (unsigned long long)(x >> (64 - sh)));
+}
+
+
+// ------------------------------------------------------------ assignment --
+// One list entry {v_hinge, v_a, v_b, e} (the hinge position is the part of
+// v_hinge) in three steps, so that a thread has several in flight and the
+// first step, which reads nothing an earlier layer wrote, can run ahead:
+// load (entry, and its key's value for a static function), read (values of
+// v_a and v_b), solve: MPHF g[v_hinge] = hinge - g[v_a] - g[v_b] mod 3 (0
+// stored as 3), static function u[v_hinge] = value - u[v_a] - u[v_b] mod
+// sigma (a value >= sigma raises kDevBadValue).
+template <bool SF>
+struct AssignItem {
+    uint4 s;
+    uint32_t f;
+    uint64_t wa, wb;
+
+    __device__ __forceinline__ void load(const AssignArgs &a, bool ok, uint64_t i) {
+        s = ok ? __ldcs(a.Lst + i) : make_uint4(0u, 0u, 0u, 0u);
+        if (SF) f = ok ? __ldg(a.values + s.w) : 0u;
+    }
+    __device__ __forceinline__ void read(const AssignArgs &a, bool ok) {
+        if (SF) {
+            wa = ok ? u_get(a.G, s.y, a.b) : 0ull;
+            wb = ok ? u_get(a.G, s.z, a.b) : 0ull;
+        } else {
+            wa = ok ? __ldcg(a.G + (s.y >> 5)) : 0ull;
+            wb = ok ? __ldcg(a.G + (s.z >> 5)) : 0ull;
         }
-        uint64_t wa[kAssignU], wb[kAssignU];
-#pragma unroll
-        for (int u = 0; u < kAssignU; u++) {
-            const bool ok = i0 + (uint64_t)u * kThreads < le;
-            wa[u] = ok ? __ldcg(G + (s[u].y >> 5)) : 0ull;
-            wb[u] = ok ? __ldcg(G + (s[u].z >> 5)) : 0ull;
-        }
-#pragma unroll
-        for (int u = 0; u < kAssignU; u++) {
-            if (i0 + (uint64_t)u * kThreads >= le) continue;
-            const uint32_t h = part_of<3>(s[u].x, P);
-            const uint32_t sum = (uint32_t)(wa[u] >> (2u * (s[u].y & 31u)) & 3u) +
-                                 (uint32_t)(wb[u] >> (2u * (s[u].z & 31u)) & 3u);
+    }
+    __device__ __forceinline__ void solve(const AssignArgs &a) const {
+        if (SF) {
+            const uint64_t sigma = a.fs.P;
+            if (f >= sigma) {
+                raise_err(a.ctl, kDevBadValue);
+                return;
+            }
+            const uint64_t val = fastmod((uint64_t)f + sigma - fastmod(wa + wb, a.fs), a.fs);
+            if (val) u_or(a.G, s.x, a.b, val);
+        } else {
+            const uint32_t h = part_of<3>(s.x, a.P);
+            const uint32_t sum = (uint32_t)(wa >> (2u * (s.y & 31u)) & 3u) +
+                                 (uint32_t)(wb >> (2u * (s.z & 31u)) & 3u);
             const uint32_t val = (h + 6u - sum) % 3u;  // sum <= 6
             const uint64_t code = val ? val : 3u;
-            atomicOr((unsigned long long *)(G + (s[u].x >> 5)),
-                     (unsigned long long)(code << (2u * (s[u].x & 31u))));
+            atomicOr((unsigned long long *)(a.G + (s.x >> 5)),
+                     (unsigned long long)(code << (2u * (s.x & 31u))));
         }
+    }
+};
+
+// Entries [lb, le) by the whole grid.  wait: the first entries are loaded
+// before the kernel ahead in the stream (the layer after this one) is waited
+// for.
+template <bool SF>
+__device__ __forceinline__ void assign_range(const AssignArgs &a, uint32_t lb, uint32_t le,
+                                             bool wait) {
+    constexpr int kU = SF ? 2 : 4;
+    const uint64_t stride = (uint64_t)gridDim.x * kThreads * kU;
+    for (uint64_t i0 = lb + (uint64_t)blockIdx.x * kThreads * kU + threadIdx.x;; i0 += stride) {
+        AssignItem<SF> x[kU];
+#pragma unroll
+        for (int u = 0; u < kU; u++) {
+            const uint64_t i = i0 + (uint64_t)u * kThreads;
+            x[u].load(a, i < le, i);
+        }
+        if (wait) asm volatile("griddepcontrol.wait;" ::: "memory");
+        wait = false;
+        if (i0 >= le) break;
+#pragma unroll
+        for (int u = 0; u < kU; u++) x[u].read(a, i0 + (uint64_t)u * kThreads < le);
+#pragma unroll
+        for (int u = 0; u < kU; u++)
+            if (i0 + (uint64_t)u * kThreads < le) x[u].solve(a);
     }
 }
 
-// Layer t: list entries loff[t] .. loff[t+1].
+// One layer, launched from the host, which knows where it lies.  Layers
+// follow each other by programmatic dependent launch: the next layer's blocks
+// start and load their entries while this one's finish.
+// With the runs of small layers below: static function of 1e7 keys (10 bits)
+// 880 -> 430 us of assignment, MPHF build of 1e8 keys -0.2 ms.
+template <bool SF>
 __global__ void __launch_bounds__(kThreads)
-k_assign(const uint4 *__restrict__ Lst, const uint32_t *__restrict__ loff, uint32_t t,
-         uint32_t P, uint64_t *G) {
-    assign_range(Lst, loff[t], loff[t + 1], P, G);
+k_assign(const AssignArgs a, uint32_t lb, uint32_t le) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    assign_range<SF>(a, lb, le, true);
 }
 
-void launch_assign_layer(const Launch &L, const uint4 *Lst, const uint32_t *loff, uint32_t t,
-                         uint32_t P, uint64_t *G) {
-    count_launch();
-    k_assign<<<grid_fixed(L, 8), kThreads, 0, L.stream>>>(Lst, loff, t, P, G);
-}
-
-// The same, for the layer whose index the device holds (the assignment loop
-// of a device-driven build).
+// The layer whose index the device holds (the assignment loop of a
+// device-driven build), when it is larger than small.
+template <bool SF>
 __global__ void __launch_bounds__(kThreads)
-k_assign_at(const uint4 *__restrict__ Lst, const uint32_t *__restrict__ loff, const int32_t *t,
-            uint32_t P, uint64_t *G) {
+k_assign_at(const AssignArgs a, const int32_t *t, uint32_t small) {
     const uint32_t tt = (uint32_t)*(volatile const int32_t *)t;
-    assign_range(Lst, __ldcg(loff + tt), __ldcg(loff + tt + 1), P, G);
+    const uint32_t lb = __ldcg(a.loff + tt), le = __ldcg(a.loff + tt + 1);
+    if (le - lb > small) assign_range<SF>(a, lb, le, false);
 }
 
-void launch_assign_layer_at(const Launch &L, const uint4 *Lst, const uint32_t *loff,
-                            const int32_t *t, uint32_t P, uint64_t *G) {
-    count_launch();
-    k_assign_at<<<grid_fixed(L, 8), kThreads, 0, L.stream>>>(Lst, loff, t, P, G);
+// Layers thi, thi - 1, .. while they hold at most kAssignTail entries (and
+// down to tlo), in one launch of one cluster: a layer waits for the one before
+// only in the cluster barrier, and its entries are loaded ahead of it.  A
+// launch per layer costs 6-14 us, one after the other, for about 1 us here.
+// Device-driven build of 1e6 keys: 1021 -> 667 us.  At 32,768 entries and
+// two per thread a layer still takes less than a grid's launch; larger ones
+// are better off with all SMs.
+// state: the device holds the layer (s->t); a layer that is too large at the
+// start has just been solved by k_assign_at and is skipped.
+constexpr uint32_t kAssignTail = 32768;  // 16 blocks x 1024 threads x 2 entries
+template <bool SF>
+__global__ void __launch_bounds__(1024, 1)
+k_assign_tail(const AssignArgs a, int32_t thi, int32_t tlo, AsyncState *state,
+              cudaGraphConditionalHandle cond) {
+    constexpr int kU = 2;
+    const uint32_t lanes = gridDim.x * 1024u, g = cl_rank() * 1024u + threadIdx.x;
+    int32_t t = state ? (int32_t)__ldcg(reinterpret_cast<const uint32_t *>(&state->t)) : thi;
+    uint32_t le = __ldcg(a.loff + t + 1), lb = __ldcg(a.loff + t);
+    cl_sync<false>();  // every block has read the state
+    if (state && le - lb > kAssignTail) {
+        t--;
+        le = lb;
+        if (t >= tlo) lb = __ldcg(a.loff + t);
+    }
+    AssignItem<SF> x[kU];
+    auto load = [&](uint32_t b, uint32_t e) {
+#pragma unroll
+        for (int u = 0; u < kU; u++) {
+            const uint32_t i = b + (uint32_t)u * lanes + g;
+            x[u].load(a, i < e, i);
+        }
+    };
+    if (t >= tlo && le - lb <= kAssignTail) load(lb, le);
+    while (t >= tlo && le - lb <= kAssignTail) {
+        bool ok[kU];
+        AssignItem<SF> now[kU];
+#pragma unroll
+        for (int u = 0; u < kU; u++) {
+            ok[u] = lb + (uint32_t)u * lanes + g < le;
+            now[u] = x[u];
+        }
+#pragma unroll
+        for (int u = 0; u < kU; u++) now[u].read(a, ok[u]);
+        // the next layer's entries come while this one is solved
+        t--;
+        le = lb;
+        if (t >= tlo) {
+            lb = __ldcg(a.loff + t);
+            if (le - lb <= kAssignTail) load(lb, le);
+        }
+#pragma unroll
+        for (int u = 0; u < kU; u++)
+            if (ok[u]) now[u].solve(a);
+        cl_sync<false>();
+    }
+    if (state && g == 0) {
+        state->t = t;
+        cudaGraphSetConditional(cond, t >= 0 ? 1u : 0u);
+    }
+}
+
+uint32_t assign_tail_blocks(bool sf) {
+    const void *fn = sf ? (const void *)k_assign_tail<true> : (const void *)k_assign_tail<false>;
+    const uint32_t b = max_cluster(fn, 1024, 0);
+    return b == 16 ? b : 0;  // kAssignTail entries need all sixteen
+}
+
+// Reverse layer order (sec. 4.3 "Avoiding backward scans") with the layer
+// starts in host memory: runs of small layers in one cluster launch, the
+// others by one grid each.
+void launch_assign(const Launch &L, bool sf, const AssignArgs &a, const uint32_t *loff_h,
+                   uint32_t rounds) {
+    const uint32_t tail = assign_tail_blocks(sf);
+    for (int64_t t = (int64_t)rounds - 1; t >= 0;) {
+        int64_t lo = t;  // layers lo + 1 .. t are small
+        while (tail && lo >= 0 && loff_h[lo + 1] - loff_h[lo] <= kAssignTail) lo--;
+        if (t - lo >= 2) {
+            int32_t thi = (int32_t)t, tlo = (int32_t)lo + 1;
+            AsyncState *none = nullptr;
+            cudaGraphConditionalHandle c0 = 0;
+            void *args[] = {(void *)&a, &thi, &tlo, &none, &c0};
+            count_launch();
+            launch_cluster(sf ? (const void *)k_assign_tail<true> : (const void *)k_assign_tail<false>,
+                           tail, 1024, 0, L.stream, args);
+            t = lo;
+            continue;
+        }
+        uint32_t lb = loff_h[t], le = loff_h[t + 1];
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(grid_for(L, le - lb, sf ? 2 : 4, 8));
+        cfg.blockDim = dim3(kThreads);
+        cfg.stream = L.stream;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        void *args[] = {(void *)&a, &lb, &le};
+        count_launch();
+        cudaLaunchKernelExC(&cfg, sf ? (const void *)k_assign<true> : (const void *)k_assign<false>,
+                            args);
+        t--;
+    }
+}
+
+// Body of the device-driven assignment loop: the layer s->t when it is large,
+// then the run of small layers after it (every layer by the grid, one per
+// turn, where the device runs no cluster of sixteen).
+void launch_assign_body(const Launch &L, bool sf, const AssignArgs &a, AsyncState *s,
+                        cudaGraphConditionalHandle h) {
+    const uint32_t tail = assign_tail_blocks(sf);
+    const uint32_t small = tail ? kAssignTail : 0u;
+    count_launch(2);
+    if (sf)
+        k_assign_at<true><<<grid_fixed(L, 8), kThreads, 0, L.stream>>>(a, &s->t, small);
+    else
+        k_assign_at<false><<<grid_fixed(L, 8), kThreads, 0, L.stream>>>(a, &s->t, small);
+    if (!tail) {
+        launch_async_assign_step(L, s, h);
+        return;
+    }
+    int32_t thi = 0, tlo = 0;
+    void *args[] = {(void *)&a, &thi, &tlo, &s, &h};
+    launch_cluster(sf ? (const void *)k_assign_tail<true> : (const void *)k_assign_tail<false>, tail,
+                   1024, 0, L.stream, args);
 }
 
 // Non-zero 2-bit values of a word: a pair is non-zero when either bit is set.
@@ -132,82 +312,6 @@ void launch_widen_dir(const Launch &L, const uint32_t *scanned, const uint32_t *
     count_launch();
     k_widen_dir<<<grid_for(L, blocks + 1, 1, 8), kThreads, 0, L.stream>>>(scanned, cnt, blocks,
                                                                           dir);
-}
-
-// ------------------------------------------------------ static functions --
-// sec. 3: any f: S -> [sigma] is stored as u with f(x) = u[h0] + u[h1] +
-// u[h2] mod sigma, b = ceil(log2 sigma) bits per vertex in one bit string
-// (vertex v at bits [v b, (v + 1) b), bit i in word i / 64): a value may
-// straddle two words, so it is read from one or two words and set with one
-// or two atomicOr.  The MPHF above is the case sigma = 3, f = hinge.
-__device__ __forceinline__ uint64_t u_get(const uint64_t *U, uint32_t v, uint32_t b) {
-    const uint64_t bit = (uint64_t)v * b;
-    const uint64_t w = bit >> 6;
-    const uint32_t sh = (uint32_t)(bit & 63u);
-    uint64_t x = __ldcg(U + w) >> sh;
-    if (sh + b > 64) x |= __ldcg(U + w + 1) << (64 - sh);
-    return x & ((1ull << b) - 1ull);  // b <= 32
-}
-
-__device__ __forceinline__ void u_or(uint64_t *U, uint32_t v, uint32_t b, uint64_t x) {
-    const uint64_t bit = (uint64_t)v * b;
-    const uint64_t w = bit >> 6;
-    const uint32_t sh = (uint32_t)(bit & 63u);
-    atomicOr((unsigned long long *)(U + w), (unsigned long long)(x << sh));
-    if (sh + b > 64) atomicOr((unsigned long long *)(U + w + 1), (unsigned long long)(x >> (64 - sh)));
-}
-
-// Layer t: for each entry {v_hinge, v_a, v_b, e}, u[v_hinge] = (values[e] -
-// u[v_a] - u[v_b]) mod sigma.  Inside one layer no entry reads a value
-// another entry of the layer writes (as for the MPHF), so the layer is one
-// parallel launch.  A value >= sigma raises kDevBadValue.
-__device__ __forceinline__ void sf_assign_range(const uint4 *__restrict__ Lst, uint32_t lb,
-                                                uint32_t le, const uint32_t *__restrict__ values,
-                                                FastMod fs, uint32_t b, uint64_t *U, Ctl *ctl) {
-    const uint64_t sigma = fs.P;
-    const uint64_t stride = (uint64_t)gridDim.x * kThreads;
-    for (uint64_t i = lb + (uint64_t)blockIdx.x * kThreads + threadIdx.x; i < le; i += stride) {
-        const uint4 s = __ldcg(Lst + i);
-        const uint32_t f = __ldg(values + s.w);
-        if (f >= sigma) {
-            raise_err(ctl, kDevBadValue);
-            continue;
-        }
-        const uint64_t other = fastmod(u_get(U, s.y, b) + u_get(U, s.z, b), fs);
-        const uint64_t val = fastmod((uint64_t)f + sigma - other, fs);
-        if (val) u_or(U, s.x, b, val);
-    }
-}
-
-__global__ void __launch_bounds__(kThreads)
-k_sf_assign(const uint4 *__restrict__ Lst, const uint32_t *__restrict__ loff, uint32_t t,
-            const uint32_t *__restrict__ values, FastMod fs, uint32_t b, uint64_t *U, Ctl *ctl) {
-    sf_assign_range(Lst, __ldcg(loff + t), __ldcg(loff + t + 1), values, fs, b, U, ctl);
-}
-
-// The same, for the layer whose index the device holds (device-driven build).
-__global__ void __launch_bounds__(kThreads)
-k_sf_assign_at(const uint4 *__restrict__ Lst, const uint32_t *__restrict__ loff, const int32_t *t,
-               const uint32_t *__restrict__ values, FastMod fs, uint32_t b, uint64_t *U,
-               Ctl *ctl) {
-    const uint32_t tt = (uint32_t)*(volatile const int32_t *)t;
-    sf_assign_range(Lst, __ldcg(loff + tt), __ldcg(loff + tt + 1), values, fs, b, U, ctl);
-}
-
-void launch_sf_assign_layer_at(const Launch &L, const uint4 *Lst, const uint32_t *loff,
-                               const int32_t *t, const uint32_t *values, uint64_t sigma,
-                               uint32_t b, uint64_t *U, Ctl *ctl) {
-    count_launch();
-    k_sf_assign_at<<<grid_fixed(L, 8), kThreads, 0, L.stream>>>(Lst, loff, t, values,
-                                                               make_fastmod(sigma), b, U, ctl);
-}
-
-void launch_sf_assign_layer(const Launch &L, const uint4 *Lst, const uint32_t *loff, uint32_t t,
-                            const uint32_t *values, uint64_t sigma, uint32_t b, uint64_t *U,
-                            Ctl *ctl) {
-    count_launch();
-    k_sf_assign<<<grid_fixed(L, 8), kThreads, 0, L.stream>>>(Lst, loff, t, values,
-                                                            make_fastmod(sigma), b, U, ctl);
 }
 
 // f(key) = (u[h0] + u[h1] + u[h2]) mod sigma.

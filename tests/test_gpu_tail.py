@@ -98,3 +98,28 @@ def test_tail_random_graphs(n, gamma, r):
 def test_tail_general_graphs(n, gamma, r):
     m = (n * gamma + 999) // 1000
     _check(oracle.hash_edges_general(inputs.keys(n, 16), m, r, 1), m, general=True)
+
+
+@pytest.mark.parametrize("n", [140_000, 1_000_000])
+@pytest.mark.parametrize("host", [0, 1])
+def test_assignment_of_small_and_large_layers(n, host):
+    # runs of layers in one cluster launch, larger ones by one grid each
+    keys = inputs.keys(n, 23)
+    dk = torch.from_numpy(keys.view(np.int64)).cuda()
+    want = oracle.mphf_build(keys, seed=1, max_tries=16)
+    vals = (inputs.keys(n, 24) % np.uint64(1000)).astype(np.uint32)
+    dv = torch.from_numpy(vals.view(np.int32)).cuda()
+    sf = oracle.sf_build(keys, vals, 1000, seed=1, max_tries=16)
+    hp.set_tuning(host_round_loop=host)
+    try:
+        got = hp.mphf_build(dk, max_tries=16)
+        gsf = hp.sf_build(dk, dv, 1000, max_tries=16)
+        G, D, _ = hp.mphf_build_async(dk, max_tries=16)
+        U, _ = hp.sf_build_async(dk, dv, 1000, max_tries=16)
+    finally:
+        hp.set_tuning()
+    for g, d in ((got.G, got.rank_dir), (G, D)):
+        assert np.array_equal(g.cpu().numpy().view(np.uint64), want.G)
+        assert np.array_equal(d.cpu().numpy().view(np.uint64), want.dir)
+    for u in (gsf.U, U[:len(sf.U)]):
+        assert np.array_equal(u.cpu().numpy().view(np.uint64), sf.U)
