@@ -89,10 +89,12 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
 }
 
 // Remainder by a runtime divisor P < 2^32 with a precomputed reciprocal
-// (Barrett reduction, P. Barrett, CRYPTO 1986).  With M = floor((2^64-1)/P)
-// the estimate q = floor(x M / 2^64) satisfies Q - 2 <= q <= Q for the true
-// quotient Q = floor(x / P), so x - q P lies in [0, 3P) and at most two
-// corrective subtractions give x mod P exactly.
+// (Barrett reduction, P. Barrett, CRYPTO 1986).  With M = floor((2^64-1)/P) >=
+// 2^64/P - 1 the product x M / 2^64 lies above x/P - 1, so its floor q is the
+// true quotient or one less: x - q P lies in [0, 2P) and one corrective
+// subtraction gives x mod P exactly.  Up to P = 2^31 that range fits 32 bits:
+// the low words suffice, and the unsigned minimum of r and r - P picks the
+// one that did not wrap.
 struct FastMod {
     uint64_t P;
     uint64_t M;
@@ -101,11 +103,13 @@ struct FastMod {
 inline FastMod make_fastmod(uint64_t P) { return FastMod{P, P ? (~0ull) / P : 0}; }
 
 __device__ __forceinline__ uint64_t fastmod(uint64_t x, const FastMod f) {
-    uint64_t q = __umul64hi(x, f.M);
-    uint64_t r = x - q * f.P;
-    if (r >= f.P) r -= f.P;
-    if (r >= f.P) r -= f.P;
-    return r;
+    const uint64_t q = __umul64hi(x, f.M);
+    if (f.P <= 0x80000000ull) {  // the same in every thread of a launch
+        const uint32_t p = (uint32_t)f.P, r = (uint32_t)x - (uint32_t)q * p;
+        return min(r, r - p);
+    }
+    const uint64_t r = x - q * f.P;
+    return r >= f.P ? r - f.P : r;
 }
 
 // Control block and parameters of the large-n MPHF build (large.cu): 64-bit

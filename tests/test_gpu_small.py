@@ -128,3 +128,33 @@ def test_small_build_seeds_past_one_launch():
                                    max_tries=130)):
         with pytest.raises(hp.HpeelError, match="RETRIES_EXHAUSTED.*seeds 1..130"):
             fn()
+
+
+@pytest.mark.parametrize("n", [1, 3, 100, 330, 341, 350, 416, 417, 1000, 4097, 200_003])
+def test_lookup_sectors_equal_the_word_path(n):
+    # the sector form needs a 32-byte aligned G; an unaligned copy takes the
+    # word form: equal on the set (a bijection) and on other keys, whatever the
+    # last block holds
+    keys = inputs.keys(n, 27)
+    dk = _dev64(keys)
+    b = hp.mphf_build(dk, max_tries=64)
+    seed = b.stats["seed_used"]
+    odd = torch.empty(b.G.numel() + 4, dtype=torch.int64, device="cuda")
+    other = _dev64(inputs.keys(20_000, 28))
+    got = hp.mphf_lookup(dk, seed, b.m, b.G, b.rank_dir).cpu().numpy()
+    assert np.array_equal(np.sort(got), np.arange(n))
+    for q in (dk, other):
+        a = hp.mphf_lookup(q, seed, b.m, b.G, b.rank_dir)
+        for shift in (1, 2, 3):
+            G = odd[shift:shift + b.G.numel()]
+            G.copy_(b.G)
+            assert torch.equal(a, hp.mphf_lookup(q, seed, b.m, G, b.rank_dir))
+
+
+@pytest.mark.parametrize("m", [1, 2, (1 << 31) - 1, 1 << 31, (1 << 31) + 1, (1 << 32) - 1])
+def test_remainders_about_2_to_the_31(m):
+    # hashes into [0, m): the 32-bit and the 64-bit form of the remainder
+    keys = np.concatenate([inputs.keys(20_000, 31), np.arange(64, dtype=np.uint64),
+                           ~np.arange(64, dtype=np.uint64)])
+    got = hp.hash_edges(_dev64(keys), m, 3, 1, general=True).cpu().numpy().view(np.uint32)
+    assert np.array_equal(got, oracle.hash_edges_general(keys, m, 3, 1))
