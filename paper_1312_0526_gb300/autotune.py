@@ -19,7 +19,8 @@ from . import _build_dir
 CACHE = os.path.join(_build_dir(), "autotune.json")
 _lock = threading.Lock()
 
-CANDIDATES = [
+# {}: the library's own launches by size class; the others: one shape for all
+CANDIDATES = [{}] + [
     {"threads": t, "ctas_per_sm": c}
     for t in (128, 256, 512)
     for c in (1, 2, 3, 4, 6, 8)

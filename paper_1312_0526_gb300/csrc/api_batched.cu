@@ -16,6 +16,7 @@ namespace {
 
 struct BatchPlan {
     uint32_t threads, ctas_per_sm, smem_bytes, smem_rounds, global16_rounds, grid;
+    uint32_t class_smem;  // shared memory of an SM when the launches go by size class, else 0
     size_t sched, next, words, scanned, tmp, scratch, total;
 };
 
@@ -29,6 +30,10 @@ hpeel_status batch_plan(uint32_t B, uint32_t gamma_milli, const hpeel_batch_tuni
         d.smem_per_sm = 233472;
         d.smem_optin = 232448;
     }
+    // no shape given: launches by size class, with global regions for two
+    // blocks per SM
+    const bool classes = !tu || (!tu->threads && !tu->ctas_per_sm && !tu->smem_bytes);
+    p->class_smem = classes ? (uint32_t)d.smem_per_sm : 0u;
     p->threads = tu && tu->threads ? tu->threads : 256u;
     p->ctas_per_sm = tu && tu->ctas_per_sm ? tu->ctas_per_sm : 2u;
     if (p->threads % 32 || p->threads < 64 || p->threads > 1024)
@@ -47,7 +52,8 @@ hpeel_status batch_plan(uint32_t B, uint32_t gamma_milli, const hpeel_batch_tuni
     const int per = d.smem_per_sm / (int)p->ctas_per_sm - 1024 - 64;
     uint32_t smem = tu && tu->smem_bytes ? tu->smem_bytes : (uint32_t)std::max(per, 0) & ~15u;
     smem = std::min<uint32_t>(smem, (uint32_t)d.smem_optin);
-    p->smem_bytes = smem;
+    // less the kernel's static shared memory, which counts against the limit
+    p->smem_bytes = classes ? (uint32_t)d.smem_optin - 64u : smem;
     p->grid = (uint32_t)d.sms * p->ctas_per_sm;
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -56,7 +62,7 @@ hpeel_status batch_plan(uint32_t B, uint32_t gamma_milli, const hpeel_batch_tuni
         return o;
     };
     p->sched = take(4 * (size_t)B + 4);
-    p->next = take(4);
+    p->next = take(kBatchCtlBytes);
     p->words = take(4 * (size_t)B + 4);
     p->scanned = take(4 * (size_t)B + 4);
     p->tmp = take(4 * scan_tmp_words(B));
@@ -129,9 +135,10 @@ hpeel_status hpeel_peel_batched(const uint64_t *d_keys, const uint64_t *d_bucket
     ProfScope ps(L, "batched");
     launch_batched(L, d_keys, d_bucket_off, B, gamma_milli, d_order, d_bucket_rounds,
                    d_bucket_status, d_G, d_G_off, p.threads, p.grid, p.smem_bytes,
-                   p.smem_rounds, p.global16_rounds,
+                   p.smem_rounds, p.global16_rounds, p.class_smem,
                    reinterpret_cast<uint32_t *>(ws + p.sched),
-                   reinterpret_cast<uint32_t *>(ws + p.next), ws + p.scratch);
+                   reinterpret_cast<uint32_t *>(ws + p.next),
+                   reinterpret_cast<uint32_t *>(ws + p.words), ws + p.scratch);
     return check_launch("batched");
 }
 

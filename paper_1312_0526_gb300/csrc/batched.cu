@@ -4,26 +4,28 @@
 // workarounds": one small hypergraph per bucket); bucket b hashes its keys
 // with seed b into a 3-partite hypergraph of m_b = 3 ceil(ceil(gamma n_b)/3)
 // vertices and is peeled on its own.  One CTA takes one bucket at a time
-// from a shared counter (work stealing over a largest-first schedule) and
-// runs the whole path for it, block-synchronous:
+// from a shared counter (work stealing over a largest-first schedule, one
+// launch per size class unless the caller gives a shape) and runs the whole
+// path for it, block-synchronous:
 //   hash + AddEdge (sec. 3, 4.1), round 0 scan, rounds with the claims of
 //   round t+1 made by the deletions of round t (sec. 4.2; same scheme as the
 //   single-graph path), the canonical order (layers ascending by round, edge
-//   ids ascending inside a layer, 2-core edges last) by a stable one-warp
-//   counting pass, and optionally the MWHC g values (sec. 3, layers last to
+//   ids ascending inside a layer, 2-core edges last) by a stable counting pass, and optionally the MWHC g values (sec. 3, layers last to
 //   first).
 // A bucket's state lives in shared memory when it fits: vertex records of 32
 // bits (degree in the low 16, sum of incident local edge ids mod 2^16 in the
 // high 16; a bucket in shared memory has far fewer than 2^16 edges, so the
 // degree never carries into the sum), claim words, the layers as 16-bit local
-// edge ids, the layer table and the g values -- no edge rows: an edge's
-// vertices are hashed again from its key (read through the cache) when a
-// round or the assignment needs them, which leaves about 11 bytes of shared
-// memory per key.  Larger buckets use a per-CTA region of the workspace,
+// edge ids, the layer table and the g values, about 9 bytes per key; when 6
+// more fit, the edges' vertices too (2,000-key buckets: 128 -> 172 keys per us
+// and SM, with the order pass on all warps), else an edge's vertices are hashed
+// again from its key (read through the cache) when a round or the assignment
+// needs them.  Larger buckets use a per-CTA region of the workspace,
 // with 32-bit records too unless the bucket has 2^16 - 1 edges or more.  No
 // block waits on another; the only cross-block state is the bucket counter.
 #include <algorithm>
 
+#include "cluster.cuh"
 #include "kernels.cuh"
 
 namespace hp {
@@ -102,6 +104,7 @@ struct BucketState {
     uint32_t *loff;  // [rcap + 2] layer starts
     uint32_t *cnt;   // [rcap + 2] running starts of the order pass
     uint32_t *G;     // [ceil(m / 16)] 2-bit g values (MPHF)
+    uint16_t *V;     // [3][n] the edges' vertices, each in its part, or null (hashed again)
     uint32_t rcap;   // rounds the loff table holds
 };
 
@@ -111,7 +114,10 @@ struct BatchArgs {
     uint32_t B;
     uint32_t gamma_milli;
     const uint32_t *sched;    // processing order of the buckets
+    const uint32_t *range;    // this launch's first and end place in sched, or null (all B)
     uint32_t *next;           // work-stealing counter
+    uint32_t *late;           // null, or where a bucket goes that does not fit this launch's
+    uint32_t *late_count;     //   shared memory (a class launch has no global regions)
     uint32_t *order;          // [total] per-bucket canonical order (local ids)
     uint32_t *rounds;         // [B] or null
     uint32_t *status;         // [B] or null: 0 peeled, 1 2-core left, 2 too large
@@ -129,13 +135,16 @@ __host__ __device__ inline size_t a16(size_t x) { return (x + 15) & ~(size_t)15;
 // Bytes of one bucket's state with records of rec_bytes and a loff table of
 // rcap + 2 entries.
 __host__ __device__ inline size_t bucket_bytes(uint32_t n, uint32_t m, uint32_t rec_bytes,
-                                               uint32_t claim_bytes, uint32_t rcap) {
+                                               uint32_t claim_bytes, uint32_t rcap,
+                                               bool verts = false) {
     return a16((size_t)m * rec_bytes) + a16((size_t)n * claim_bytes) + a16((size_t)n * 2) +
-           2 * a16(((size_t)rcap + 2) * 4) + a16(((size_t)m + 15) / 16 * 4);
+           2 * a16(((size_t)rcap + 2) * 4) + a16(((size_t)m + 15) / 16 * 4) +
+           (verts ? a16((size_t)n * 6) : 0);
 }
 
 template <typename T, typename C>
-__device__ BucketState<T, C> carve(char *base, uint32_t n, uint32_t m, uint32_t rcap) {
+__device__ BucketState<T, C> carve(char *base, uint32_t n, uint32_t m, uint32_t rcap,
+                                   bool verts = false) {
     BucketState<T, C> s;
     size_t o = 0;
     s.rec = reinterpret_cast<T *>(base + o);
@@ -149,6 +158,8 @@ __device__ BucketState<T, C> carve(char *base, uint32_t n, uint32_t m, uint32_t 
     s.cnt = reinterpret_cast<uint32_t *>(base + o);
     o += a16(((size_t)rcap + 2) * 4);
     s.G = reinterpret_cast<uint32_t *>(base + o);
+    o += a16(((size_t)m + 15) / 16 * 4);
+    s.V = verts ? reinterpret_cast<uint16_t *>(base + o) : nullptr;
     s.rcap = rcap;
     return s;
 }
@@ -167,10 +178,25 @@ __device__ __forceinline__ void cta_append(uint32_t *cursor, uint16_t *list, uin
     if (pred) list[list_base + base + __popc(ballot & ((1u << lane) - 1u))] = (uint16_t)v;
 }
 
+// Two candidates per lane, one reservation.
+__device__ __forceinline__ void cta_append2(uint32_t *cursor, uint16_t *list, uint32_t list_base,
+                                            const bool (&pred)[2], const uint32_t (&v)[2]) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, pred[0]);
+    const uint32_t b1 = __ballot_sync(0xFFFFFFFFu, pred[1]);
+    if (!(b0 | b1)) return;
+    uint32_t base = 0;
+    if (lane == 0) base = atomicAdd(cursor, (uint32_t)(__popc(b0) + __popc(b1)));
+    base = list_base + __shfl_sync(0xFFFFFFFFu, base, 0);
+    const uint32_t lt = (1u << lane) - 1u;
+    if (pred[0]) list[base + __popc(b0 & lt)] = (uint16_t)v[0];
+    if (pred[1]) list[base + __popc(b0) + __popc(b1 & lt)] = (uint16_t)v[1];
+}
+
 // The whole path for one bucket.  Every thread of the block calls it.
 // Returns false (writing nothing) when the bucket needs more rounds than its
 // layer table holds; the caller reruns it with a larger table.
-template <typename T, typename C>
+template <typename T, typename C, bool VERTS>
 __device__ bool run_bucket(const BatchArgs &a, uint32_t b, BucketState<T, C> s, uint32_t n,
                            uint32_t m, uint32_t *sh) {
     const uint32_t kUnc = unclaimed<C>();
@@ -198,7 +224,10 @@ __device__ bool run_bucket(const BatchArgs &a, uint32_t b, BucketState<T, C> s, 
         uint32_t v[3];
         bucket_edge(__ldg(keys + e), seed, fm, P, v);
 #pragma unroll
-        for (int j = 0; j < 3; j++) atomicAdd(s.rec + v[j], V::unit(e));
+        for (int j = 0; j < 3; j++) {
+            atomicAdd(s.rec + v[j], V::unit(e));
+            if (VERTS) s.V[(uint32_t)j * n + e] = (uint16_t)(v[j] - (uint32_t)j * P);
+        }
     }
     __syncthreads();
     // round 0
@@ -244,24 +273,32 @@ __device__ bool run_bucket(const BatchArgs &a, uint32_t b, BucketState<T, C> s, 
             if (i < le) {
                 const uint32_t e = s.L[i];
                 const uint32_t h = s.claim[e] & 3u;
-                uint32_t v[3];
-                bucket_edge(__ldg(keys + e), seed, fm, P, v);
+                const uint32_t j0 = h == 0 ? 1u : 0u, j1 = h == 2 ? 1u : 2u;
+                uint32_t x[2];
+                if (VERTS) {
+                    x[0] = s.V[j0 * n + e] + j0 * P;
+                    x[1] = s.V[j1 * n + e] + j1 * P;
+                } else {
+                    uint32_t v[3];
+                    bucket_edge(__ldg(keys + e), seed, fm, P, v);
+                    x[0] = h == 0 ? v[1] : v[0];
+                    x[1] = h == 2 ? v[1] : v[2];
+                }
+                T old[2];
+#pragma unroll
+                for (int k = 0; k < 2; k++) old[k] = atomicAdd(s.rec + x[k], (T)(0) - V::unit(e));
 #pragma unroll
                 for (int k = 0; k < 2; k++) {
-                    const int j = k + ((uint32_t)k >= h ? 1 : 0);
-                    const T old = atomicAdd(s.rec + v[j], (T)(0) - V::unit(e));
-                    if (V::deg(old) == 2u) {
-                        const uint32_t g = (V::sum(old) - e) & V::mask();
+                    if (V::deg(old[k]) == 2u) {
+                        const uint32_t g = (V::sum(old[k]) - e) & V::mask();
                         if (g < n) {
-                            take[k] = claim_min(s.claim + g, ((t + 1) << 2) | (uint32_t)j) ==
-                                      kUnc;
+                            take[k] = claim_min(s.claim + g, ((t + 1) << 2) | (k ? j1 : j0)) == kUnc;
                             f[k] = g;
                         }
                     }
                 }
             }
-            cta_append(cur, s.L, le, take[0], f[0]);
-            cta_append(cur, s.L, le, take[1], f[1]);
+            cta_append2(cur, s.L, le, take, f);
         }
         __syncthreads();
         const uint32_t next = le + *(volatile uint32_t *)cur;
@@ -275,23 +312,64 @@ __device__ bool run_bucket(const BatchArgs &a, uint32_t b, BucketState<T, C> s, 
     __syncthreads();
     uint32_t *out = a.order + key0;
     if (too_many) return false;  // block-uniform
-    // canonical order: one warp walks the edges in id order (stable), the
-    // running start of every layer in cnt[0..R], the core after them
-    if (tid < 32) {
-        const uint32_t lane = tid;
+    // canonical order.  Every warp takes a run of consecutive edges: counts
+    // per layer, the layers' starts and the counts of the lower warps give
+    // where its edges of a layer go, and a second walk places them in id order
+    // (the vertex records are dead: their space holds the counts).
+    const uint32_t nw = T_ / 32u, lane = tid & 31u, warp = tid >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    auto key_of = [&](uint32_t e) {
+        const uint32_t c = s.claim[e];
+        return c == kUnc ? R : c >> 2;
+    };
+    if ((size_t)nw * (R + 1) * 4 <= (size_t)m * sizeof(T)) {
+        uint32_t *wh = reinterpret_cast<uint32_t *>(s.rec) + warp * (R + 1);
+        for (uint32_t r = lane; r <= R; r += 32) wh[r] = 0;
+        __syncwarp();
+        const uint32_t run = ((n + nw - 1) / nw + 31u) & ~31u;
+        const uint32_t e_lo = min(warp * run, n), e_hi = min(e_lo + run, n);
+        for (uint32_t e0 = e_lo; e0 < e_hi; e0 += 32) {
+            const uint32_t e = e0 + lane;
+            if (e < e_hi) atomicAdd(wh + key_of(e), 1u);
+        }
+        __syncthreads();
+        for (uint32_t r = tid; r <= R; r += T_) {
+            uint32_t at = r < R ? s.loff[r] : peeled;
+            uint32_t *p = reinterpret_cast<uint32_t *>(s.rec) + r;
+            for (uint32_t w = 0; w < nw; w++, p += R + 1) {
+                const uint32_t c = *p;
+                *p = at;
+                at += c;
+            }
+        }
+        __syncthreads();
+        for (uint32_t e0 = e_lo; e0 < e_hi; e0 += 32) {
+            const uint32_t e = e0 + lane;
+            const bool valid = e < e_hi;
+            const uint32_t key = valid ? key_of(e) : 0xFFFFFFFFu;
+            const uint32_t peers = __match_any_sync(0xFFFFFFFFu, key);
+            const uint32_t below = __popc(peers & lt);
+            uint32_t at = 0;
+            if (valid) {
+                at = wh[key];
+                out[at + below] = e;
+            }
+            __syncwarp();
+            if (valid && below == 0) wh[key] = at + __popc(peers);
+            __syncwarp();
+        }
+    } else if (warp == 0) {
+        // more layers than the records' space holds: one warp walks all edges,
+        // the running start of every layer in cnt[0..R]
         uint32_t *cnt = s.cnt;
         for (uint32_t r = lane; r <= R; r += 32) cnt[r] = r < R ? s.loff[r] : peeled;
         __syncwarp();
         for (uint32_t e0 = 0; e0 < n; e0 += 32) {
             const uint32_t e = e0 + lane;
             const bool valid = e < n;
-            uint32_t key = 0xFFFFFFFFu;
-            if (valid) {
-                const uint32_t c = s.claim[e];
-                key = c == kUnc ? R : (c >> 2);
-            }
+            const uint32_t key = valid ? key_of(e) : 0xFFFFFFFFu;
             const uint32_t peers = __match_any_sync(0xFFFFFFFFu, key);
-            if (valid) out[cnt[key] + __popc(peers & ((1u << lane) - 1u))] = e;
+            if (valid) out[cnt[key] + __popc(peers & lt)] = e;
             __syncwarp();
             if (valid && lane == (uint32_t)(__ffs(peers) - 1)) cnt[key] += __popc(peers);
             __syncwarp();
@@ -314,7 +392,13 @@ __device__ bool run_bucket(const BatchArgs &a, uint32_t b, BucketState<T, C> s, 
                 const uint32_t e = s.L[i];
                 const uint32_t h = s.claim[e] & 3u;
                 uint32_t v[3];
-                bucket_edge(__ldg(keys + e), seed, fm, P, v);
+                if (VERTS) {
+#pragma unroll
+                    for (int j = 0; j < 3; j++)
+                        v[j] = s.V[(uint32_t)j * n + e] + (uint32_t)j * P;
+                } else {
+                    bucket_edge(__ldg(keys + e), seed, fm, P, v);
+                }
                 uint32_t sum = 0;
 #pragma unroll
                 for (int j = 0; j < 3; j++)
@@ -342,15 +426,21 @@ __device__ bool run_bucket(const BatchArgs &a, uint32_t b, BucketState<T, C> s, 
     return true;
 }
 
-__global__ void k_batched(BatchArgs a) {
+
+// 32 registers and so 2,048 threads per SM (9.57 ms for 65,536 lognormal
+// buckets; with 56 registers 9.84, with 40 by __maxnreg__ 11.06).
+__global__ void __launch_bounds__(1024, 2) k_batched(BatchArgs a) {
     extern __shared__ __align__(16) char smem[];
     __shared__ __align__(16) uint32_t sh[8];  // sh[2..3] hold a 64-bit value
     __shared__ uint32_t s_b;
+    // the next class's blocks may start as this one's leave (see launch_batched)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     char *region = a.scratch + (size_t)blockIdx.x * a.scratch_bytes;
+    const uint32_t lo = a.range ? __ldcg(a.range) : 0u, hi = a.range ? __ldcg(a.range + 1) : a.B;
     for (;;) {
         if (threadIdx.x == 0) {
-            const uint32_t k = atomicAdd(a.next, 1u);
-            s_b = k < a.B ? a.sched[k] : 0xFFFFFFFFu;
+            const uint32_t k = lo < hi ? lo + atomicAdd(a.next, 1u) : hi;
+            s_b = k < hi ? a.sched[k] : 0xFFFFFFFFu;
         }
         __syncthreads();
         const uint32_t b = s_b;
@@ -371,22 +461,33 @@ __global__ void k_batched(BatchArgs a) {
         const uint32_t m = bucket_vertices(n, a.gamma_milli);
         const uint32_t rcap_s = min(n + 1, a.smem_rounds);
         bool done = false;
-        if (n < 0xFFFFu && bucket_bytes(n, m, 4, 2, rcap_s) <= a.smem_bytes)
-            done = run_bucket<uint32_t, uint16_t>(a, b, carve<uint32_t, uint16_t>(smem, n, m, rcap_s),
-                                                  n, m, sh);
+        if (n < 0xFFFFu) {
+            if (bucket_bytes(n, m, 4, 2, rcap_s, true) <= a.smem_bytes)
+                done = run_bucket<uint32_t, uint16_t, true>(
+                    a, b, carve<uint32_t, uint16_t>(smem, n, m, rcap_s, true), n, m, sh);
+            else if (bucket_bytes(n, m, 4, 2, rcap_s) <= a.smem_bytes)
+                done = run_bucket<uint32_t, uint16_t, false>(
+                    a, b, carve<uint32_t, uint16_t>(smem, n, m, rcap_s), n, m, sh);
+        }
+        if (!done && a.late) {
+            if (threadIdx.x == 0) a.late[atomicAdd(a.late_count, 1u)] = b;
+            continue;
+        }
         // the global region: 32-bit records and 16-bit claims when the
         // 16-bit fields hold the bucket (fewer than 2^16 - 1 edges, at most
         // global16_rounds <= kClaim16Rounds rounds), as in shared memory;
         // else 64-bit records and 32-bit claims with room for every round
         // (n + 1 layer starts)
         if (!done && n < 0xFFFFu)
-            done = run_bucket<uint32_t, uint16_t>(
+            done = run_bucket<uint32_t, uint16_t, false>(
                 a, b, carve<uint32_t, uint16_t>(region, n, m, min(n + 1, a.global16_rounds)), n,
                 m, sh);
         if (!done)
-            run_bucket<unsigned long long, uint32_t>(
+            run_bucket<unsigned long long, uint32_t, false>(
                 a, b, carve<unsigned long long, uint32_t>(region, n, m, n + 1), n, m, sh);
     }
+    // a launch ends only after the one before it
+    if (blockIdx.x == 0 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // Word offsets of the buckets' g arrays: G_off[b] = sum of ceil(m_c / 32)
@@ -415,33 +516,91 @@ void launch_batch_g_offsets(const Launch &L, const uint64_t *off, uint32_t B, ui
                                                                                G_off);
 }
 
-// Largest-first schedule: buckets by size class (log2), classes descending.
-__global__ void k_batch_schedule(const uint64_t *off, uint32_t B, uint32_t *sched,
-                                 uint32_t *next) {
-    __shared__ uint32_t cls[34];
-    for (uint32_t c = threadIdx.x; c < 34; c += blockDim.x) cls[c] = 0;
-    __syncthreads();
-    for (uint32_t b = threadIdx.x; b < B; b += blockDim.x) {
-        const uint64_t n = off[b + 1] - off[b];
-        const uint32_t c = n ? 64 - __clzll(n) : 0;  // 0..33
-        atomicAdd(&cls[c < 33 ? c : 33], 1u);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t s = 0;
-        for (int c = 33; c >= 0; c--) {
-            const uint32_t k = cls[c];
-            cls[c] = s;
-            s += k;
+// Launch classes: buckets of one size range in one launch, with the blocks per
+// SM (and so the shared memory per block) and the threads that suit them.  One
+// shape for all sizes leaves half the keys of a lognormal workload in the
+// global regions (2.01e8 keys in 65,536 buckets: 14.9 ms at 256 threads x 6
+// blocks, the best single shape).  Rates of uniform buckets (keys per us and
+// SM, with g values) at the shape chosen and at the next best: 200 keys 119 /
+// 108, 1000 182 / 159, 1500 158 / 147, 2000 152 / 141, 3500 147 / 145, 4000
+// 131 / 130, 6000 118 / 112, 8000 107 / 104, 12000 102 / 97, 24000 95 / 91,
+// 60000 (global regions) 33 / 25.
+struct BatchClass {
+    uint32_t threads, ctas;
+    bool verts;   // takes buckets whose vertices fit beside their state, or
+    int launch;   // any that fit; index of the launch (largest buckets first)
+};
+constexpr int kBatchLaunches = 9;  // 0: the global regions
+constexpr int kBatchClasses = 11;
+struct BatchShapes {
+    uint32_t smem[kBatchClasses];  // dynamic shared memory of a class's block
+    uint32_t launch[kBatchClasses];
+    bool verts[kBatchClasses];
+    uint32_t smem_rounds, gamma_milli;
+};
+// tried in this order, the first that holds the bucket takes it
+constexpr BatchClass kBatchClass[kBatchClasses] = {
+    {64, 24, true, 8},  {128, 12, true, 7}, {128, 8, true, 6},  {256, 6, true, 5},
+    {384, 4, true, 4},  {384, 3, true, 3},  {384, 4, false, 4}, {512, 2, true, 2},
+    {384, 3, false, 3}, {512, 2, false, 2}, {768, 1, false, 1}};
+
+__device__ __forceinline__ uint32_t batch_launch(const BatchShapes &s, uint32_t n) {
+    const uint32_t m = bucket_vertices(n, s.gamma_milli), rcap = min(n + 1, s.smem_rounds);
+    const size_t plain = bucket_bytes(n, m, 4, 2, rcap), verts = bucket_bytes(n, m, 4, 2, rcap, true);
+    if (n >= 0xFFFFu) return 0;
+#pragma unroll
+    for (int c = 0; c < kBatchClasses; c++)
+        if ((s.verts[c] ? verts : plain) <= s.smem[c]) return s.launch[c];
+    return 0;
+}
+
+// Schedule: buckets by launch, largest first inside a launch (quarters of an
+// octave), by one cluster.  ctl: [0 .. kBatchLaunches] the launches' starts
+// (and end), from 16 on their counters, then the late list's count and counter.
+// plain: one launch of all buckets, largest first.
+constexpr uint32_t kBatchSizes = 4 * 17 + 1;  // quarter octaves up to 2^17
+constexpr uint32_t kBatchBins = kBatchLaunches * kBatchSizes;
+constexpr uint32_t kBatchCtlNext = 16, kBatchCtlLate = 32, kBatchCtlWords = 34;
+__global__ void __launch_bounds__(1024)
+k_batch_schedule(const uint64_t *off, uint32_t B, BatchShapes shapes, uint32_t plain, uint32_t *sched,
+                 uint32_t *ctl) {
+    __shared__ uint32_t cnt[kBatchBins], total[kBatchBins], low[kBatchBins];
+    const uint32_t tid = threadIdx.x, rank = cl_rank(), blocks = gridDim.x;
+    auto bin_of = [&](uint32_t b) {
+        const uint64_t n64 = off[b + 1] - off[b];
+        const uint32_t n = (uint32_t)(n64 < 131071u ? n64 : 131071u);
+        // larger sizes in lower bins; a bucket past the limit is only reported
+        const uint32_t lg = n ? 31u - __clz(n) : 0u;
+        const uint32_t q = n ? 4u * lg + (lg >= 2 ? (n >> (lg - 2)) & 3u : 0u) + 1u : 0u;
+        const uint32_t launch = plain ? 0u : (n64 > kBatchMaxEdges ? 0u : batch_launch(shapes, n));
+        return launch * kBatchSizes + (kBatchSizes - 1u - q);
+    };
+    for (uint32_t i = tid; i < kBatchBins; i += 1024) cnt[i] = 0;
+    cl_sync<false>();
+    const uint32_t stride = blocks * 1024u, first = rank * 1024u + tid;
+    for (uint64_t b = first; b < B; b += stride) atomicAdd(&cnt[bin_of((uint32_t)b)], 1u);
+    cl_sync<false>();
+    for (uint32_t i = tid; i < kBatchBins; i += 1024) {
+        uint32_t s = 0, l = 0;
+        for (uint32_t c = 0; c < blocks; c++) {
+            if (c == rank) l = s;
+            s += cl_load<false>(cl_map<false>(smem_u32(cnt + i), c));
         }
-        *next = 0;
+        total[i] = s;
+        low[i] = l;
+    }
+    cl_sync<false>();  // the counts are read: they become cursors
+    block_scan_counts<1024>(total, cnt, kBatchBins);
+    if (rank == 0) {
+        if (tid < kBatchLaunches) ctl[tid] = cnt[tid * kBatchSizes];
+        if (tid == kBatchLaunches) ctl[tid] = B;
+        if (tid >= kBatchCtlNext && tid < kBatchCtlWords) ctl[tid] = 0;
     }
     __syncthreads();
-    for (uint32_t b = threadIdx.x; b < B; b += blockDim.x) {
-        const uint64_t n = off[b + 1] - off[b];
-        const uint32_t c = n ? 64 - __clzll(n) : 0;
-        sched[atomicAdd(&cls[c < 33 ? c : 33], 1u)] = b;
-    }
+    for (uint32_t i = tid; i < kBatchBins; i += 1024) cnt[i] += low[i];
+    __syncthreads();
+    for (uint64_t b = first; b < B; b += stride)
+        sched[atomicAdd(&cnt[bin_of((uint32_t)b)], 1u)] = (uint32_t)b;
 }
 
 // Per-CTA global region: the largest bucket at this sparsity.
@@ -467,15 +626,83 @@ void launch_batched(const Launch &L, const uint64_t *keys, const uint64_t *off, 
                     uint32_t gamma_milli, uint32_t *order, uint32_t *rounds, uint32_t *status,
                     uint64_t *G, const uint64_t *G_off, uint32_t threads, uint32_t ctas,
                     uint32_t smem_bytes, uint32_t smem_rounds, uint32_t global16_rounds,
-                    uint32_t *sched, uint32_t *next, char *scratch) {
-    count_launch();
-    k_batch_schedule<<<1, 1024, 0, L.stream>>>(off, B, sched, next);
-    BatchArgs a{keys, off, B, gamma_milli, sched, next, order, rounds, status, G, G_off,
-                scratch, batched_scratch_bytes(gamma_milli), smem_bytes, smem_rounds,
-                global16_rounds};
+                    uint32_t smem_per_sm, uint32_t *sched, uint32_t *ctl, uint32_t *late,
+                    char *scratch) {
+    const bool classes = smem_per_sm != 0;
+    BatchShapes sh{};
+    sh.smem_rounds = smem_rounds;
+    sh.gamma_milli = gamma_milli;
     smem_optin((const void *)k_batched);
-    count_launch();
-    k_batched<<<ctas, threads, smem_bytes, L.stream>>>(a);
+    // what a block may ask for, and what the SM holds of them (1 KB per block
+    // is reserved, 64 B static)
+    for (int c = 0; c < kBatchClasses; c++) {
+        sh.launch[c] = (uint32_t)kBatchClass[c].launch;
+        sh.verts[c] = kBatchClass[c].verts;
+        sh.smem[c] = classes ? std::min(smem_bytes, (smem_per_sm / kBatchClass[c].ctas - 1024 - 64) & ~15u)
+                             : 0u;
+    }
+    {
+        uint32_t plain = classes ? 0u : 1u;
+        uint32_t blocks = max_cluster((const void *)k_batch_schedule, 1024, 0);
+        if (blocks == 0) blocks = 1;
+        while (blocks > 1 && (uint64_t)(blocks / 2) * 1024u >= B) blocks /= 2;
+        void *args[] = {(void *)&off, (void *)&B, (void *)&sh, (void *)&plain, (void *)&sched,
+                        (void *)&ctl};
+        count_launch();
+        launch_cluster((const void *)k_batch_schedule, blocks, 1024, 0, L.stream, args);
+    }
+    BatchArgs a{keys, off, B, gamma_milli, sched, nullptr, ctl + kBatchCtlNext, nullptr, nullptr,
+                order, rounds, status, G, G_off, scratch, batched_scratch_bytes(gamma_milli),
+                smem_bytes, smem_rounds, global16_rounds};
+    if (!classes) {
+        count_launch();
+        k_batched<<<ctas, threads, smem_bytes, L.stream>>>(a);
+        return;
+    }
+    // The launches overlap: each lets the next one's blocks start as its own
+    // leave (programmatic dependent launch; they share nothing but the
+    // outputs, bucket by bucket), and ends only after the one before it.  The
+    // last takes the buckets that needed more rounds than their class's shared
+    // memory holds; it shares the global regions with the first, so it starts
+    // when all others have ended.
+    for (int l = 0; l <= kBatchLaunches; l++) {
+        const bool global = l == 0 || l == kBatchLaunches;
+        BatchArgs x = a;
+        uint32_t th = 1024, per = 2;
+        for (int c = 0; c < kBatchClasses && !global; c++)
+            if (kBatchClass[c].launch == l) {
+                th = kBatchClass[c].threads;
+                per = kBatchClass[c].ctas;
+                x.smem_bytes = sh.smem[c];
+            }
+        if (l < kBatchLaunches) {
+            x.range = ctl + l;
+            x.next = ctl + kBatchCtlNext + l;
+        } else {
+            x.sched = late;
+            x.range = ctl + kBatchCtlLate - 1;  // 0, the late buckets' count
+            x.next = ctl + kBatchCtlLate + 1;
+        }
+        if (global) {
+            x.smem_bytes = 0;
+        } else {
+            x.late = late;
+            x.late_count = ctl + kBatchCtlLate;
+        }
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)L.sms * per);
+        cfg.blockDim = dim3(th);
+        cfg.dynamicSmemBytes = x.smem_bytes;
+        cfg.stream = L.stream;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = l > 0 && l < kBatchLaunches ? 1 : 0;
+        void *args[] = {(void *)&x};
+        count_launch();
+        cudaLaunchKernelExC(&cfg, (const void *)k_batched, args);
+    }
 }
 
 }  // namespace hp

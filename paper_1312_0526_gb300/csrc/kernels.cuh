@@ -364,12 +364,17 @@ size_t batched_scratch_bytes(uint32_t gamma_milli);
 uint32_t batched_max_gamma_milli();
 // Most layer-table entries of a bucket with 16-bit claim words.
 uint32_t batched_claim16_rounds();
+// ctl: kBatchCtlBytes of workspace; late: B words.  smem_per_sm 0: one launch
+// of all buckets with the given shape; else the launches by size class
+// (smem_bytes: the most a block may ask for), whose global regions are
+// 2 per SM.
+constexpr size_t kBatchCtlBytes = 256;
 void launch_batched(const Launch &L, const uint64_t *keys, const uint64_t *off, uint32_t B,
                     uint32_t gamma_milli, uint32_t *order, uint32_t *rounds, uint32_t *status,
                     uint64_t *G, const uint64_t *G_off, uint32_t threads, uint32_t ctas,
                     uint32_t smem_bytes, uint32_t smem_rounds, uint32_t global16_rounds,
-                    uint32_t *sched,
-                    uint32_t *next, char *scratch);
+                    uint32_t smem_per_sm, uint32_t *sched, uint32_t *ctl, uint32_t *late,
+                    char *scratch);
 void launch_batch_g_offsets(const Launch &L, const uint64_t *off, uint32_t B, uint32_t gamma_milli,
                             uint32_t *words, uint32_t *scanned, uint32_t *tmp, uint64_t *G_off);
 
