@@ -2080,7 +2080,15 @@ hpeel_status hpeel_mphf_build_large(const uint64_t *d_keys, uint64_t n, uint64_t
         {
             ProfScope ps(L, "large_build");
             launch_fill_u32(L, reinterpret_cast<uint32_t *>(st), 2 * m, 0u);
-            launch_large_build(L, d_keys, n, s, fm, st, claim, ctl);
+            // claim words and layer list are adjacent and not in use yet
+            const size_t room_end = h_list ? lay.claim + 4 * n : lay.L + 8 * n;
+            const LargeBuildPlan bp = large_build_plan(n, P, room_end - lay.claim);
+            if (m >= tu.bucket_min_vertices && bp.per_pass) {
+                launch_large_build_bucketed(L, bp, d_keys, n, s, fm, st, ws + lay.claim, ctl);
+                launch_fill_u32(L, claim, n, 0xFFFFFFFFu);
+            } else {
+                launch_large_build(L, d_keys, n, s, fm, st, claim, ctl);
+            }
         }
         LargeParams lp{st, claim, Ll, loff, ctl, d_keys, n, m, s, fm, lay.max_rounds};
         launch_large_set_params(L, prm, lp);

@@ -317,6 +317,19 @@ void launch_layer_off_dev(const Launch &L, const uint32_t *loff, const Ctl *ctl,
 // f4: MPHF build beyond 32-bit ids (large.cu).
 RoundLaunch large_round_launch(const Launch &L, bool first);
 void launch_large_set_params(const Launch &L, LargeParams *dst, const LargeParams &v);
+// The build by vertex range: chunks of 2^kLargeChunk vertices of a part, per_pass
+// of them per pass over the keys (0: the room is too small, build directly).
+// room: cursors, then the chunks' arrays of cap 8-byte pairs.  The vertex
+// records are zeroed before, the claim words written after.
+constexpr uint32_t kLargeChunk = 22;
+struct LargeBuildPlan {
+    uint32_t chunks, per_pass;
+    uint64_t cap;
+};
+LargeBuildPlan large_build_plan(uint64_t n, uint64_t P, uint64_t room);
+void launch_large_build_bucketed(const Launch &L, const LargeBuildPlan &b, const uint64_t *keys,
+                                 uint64_t n, uint64_t seed, FastMod fm, unsigned long long *st,
+                                 char *room, LargeCtl *ctl);
 void launch_large_build(const Launch &L, const uint64_t *keys, uint64_t n, uint64_t seed,
                         FastMod fm, unsigned long long *st, uint32_t *claim, LargeCtl *ctl);
 void launch_large_assign(const Launch &L, const LargeParams *prm, uint32_t t, uint64_t *G);
