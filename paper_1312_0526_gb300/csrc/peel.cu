@@ -457,6 +457,10 @@ k_round(const RoundParams *__restrict__ prm, Ctl *__restrict__ ctl,
     const uint4 now = __ldcg(reinterpret_cast<const uint4 *>(&ctl->round));
     const uint32_t t = now.x;
     uint32_t lb = now.y, le = now.z;
+    // in a graph the round kernel stands several times in the loop's body: the
+    // ones after the last large layer have nothing to do (the same decision in
+    // every block: the state moves only when all blocks have counted in)
+    if (cond && (!now.w || le - lb <= prm->tail_max)) return;
     if (lb > le || le > n) {  // inconsistent state: report, delete nothing
         raise_err(ctl, kDevCapacity);
         lb = le;
