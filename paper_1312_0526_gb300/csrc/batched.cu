@@ -41,24 +41,27 @@ constexpr uint32_t kClaim16Rounds = 16383;
 template <typename C>
 __device__ __forceinline__ uint32_t unclaimed() { return (uint32_t)(C)~(C)0; }
 
-// atomicMin on a claim word, returning the old value
-__device__ __forceinline__ uint32_t claim_min(uint32_t *p, uint32_t v) { return atomicMin(p, v); }
-__device__ __forceinline__ uint32_t claim_min(uint16_t *p, uint32_t v) {
-    // the 32-bit word holding the half-word: compare-and-swap until the
-    // half-word is at most v (every failed swap saw another claim succeed)
+// A claim is (round << 2) | code, code 0, 1, 3 for hinge position 0, 1, 2: the
+// bitwise and of a round's claims of an edge is its smallest one, so a claim in
+// a 16-bit word is one atomicAnd on the 32-bit word around it, with no
+// compare-and-swap loop.  (All ones is no claim: a 16-bit round stays below
+// kClaim16Rounds.)  It must not touch an edge claimed in an earlier round, so
+// the word is read first: such a claim was there before the round's barrier.
+__device__ __forceinline__ uint32_t hinge_code(uint32_t j) { return j + (j >> 1); }
+__device__ __forceinline__ uint32_t hinge_of(uint32_t claim) { return (claim & 3u) - ((claim >> 1) & 1u); }
+__device__ __forceinline__ bool claim_open(const uint32_t *, uint32_t) { return true; }
+__device__ __forceinline__ bool claim_open(const uint16_t *p, uint32_t tag) {
+    const uint32_t c = *reinterpret_cast<const volatile uint16_t *>(p);
+    return c == 0xFFFFu || (c >> 2) == (tag >> 2);
+}
+// the claim before this one (call for an open claim word)
+__device__ __forceinline__ uint32_t claim_put(uint32_t *p, uint32_t tag) { return atomicMin(p, tag); }
+__device__ __forceinline__ uint32_t claim_put(uint16_t *p, uint32_t tag) {
     uint32_t *w = reinterpret_cast<uint32_t *>(reinterpret_cast<uintptr_t>(p) & ~(uintptr_t)3);
     const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(p) & 2u) * 8u;
-    uint32_t old = *reinterpret_cast<volatile uint32_t *>(w);
-    for (;;) {
-        const uint32_t cur = (old >> sh) & 0xFFFFu;
-        if (cur <= v) return cur;
-        const uint32_t got = atomicCAS(w, old, (old & ~(0xFFFFu << sh)) | (v << sh));
-        if (got == old) return cur;
-        old = got;
-    }
+    return (atomicAnd(w, ~((0xFFFFu ^ tag) << sh)) >> sh) & 0xFFFFu;
 }
 
-// Device copy of hpeel_num_vertices for r = 3.
 __device__ __forceinline__ uint32_t bucket_vertices(uint32_t n, uint32_t gamma_milli) {
     const uint64_t gn = ((uint64_t)n * gamma_milli + 999u) / 1000u;
     return (uint32_t)((gn + 2) / 3 * 3);
@@ -164,21 +167,8 @@ __device__ BucketState<T, C> carve(char *base, uint32_t n, uint32_t m, uint32_t 
     return s;
 }
 
-// Warp-aggregated append to a block-local list: slot list_base + the value
-// of a shared counter.
-__device__ __forceinline__ void cta_append(uint32_t *cursor, uint16_t *list, uint32_t list_base,
-                                           bool pred, uint32_t v) {
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t ballot = __ballot_sync(0xFFFFFFFFu, pred);
-    if (!ballot) return;
-    const uint32_t leader = __ffs(ballot) - 1;
-    uint32_t base = 0;
-    if (lane == leader) base = atomicAdd(cursor, (uint32_t)__popc(ballot));
-    base = __shfl_sync(0xFFFFFFFFu, base, leader);
-    if (pred) list[list_base + base + __popc(ballot & ((1u << lane) - 1u))] = (uint16_t)v;
-}
-
-// Two candidates per lane, one reservation.
+// Warp-aggregated append to a block-local list (slot list_base + the value of a
+// shared counter): two candidates per lane, one reservation.
 __device__ __forceinline__ void cta_append2(uint32_t *cursor, uint16_t *list, uint32_t list_base,
                                             const bool (&pred)[2], const uint32_t (&v)[2]) {
     const uint32_t lane = threadIdx.x & 31u;
@@ -192,6 +182,10 @@ __device__ __forceinline__ void cta_append2(uint32_t *cursor, uint16_t *list, ui
     if (pred[0]) list[base + __popc(b0 & lt)] = (uint16_t)v[0];
     if (pred[1]) list[base + __popc(b0) + __popc(b1 & lt)] = (uint16_t)v[1];
 }
+
+// Edges of a layer that one warp takes: one per lane (65,536 lognormal buckets,
+// 8.28 ms; layers of up to 48 8.48, 64 8.63, none 8.60).
+constexpr uint32_t kWarpLayer = 32;
 
 // The whole path for one bucket.  Every thread of the block calls it.
 // Returns false (writing nothing) when the bucket needs more rounds than its
@@ -230,25 +224,90 @@ __device__ bool run_bucket(const BatchArgs &a, uint32_t b, BucketState<T, C> s, 
         }
     }
     __syncthreads();
-    // round 0
-    for (uint32_t v0 = 0; v0 < m; v0 += T_) {
-        const uint32_t v = v0 + tid;
-        bool take = false;
-        uint32_t e = 0;
-        if (v < m) {
-            const T r = s.rec[v];
-            if (V::deg(r) == 1u && V::sum(r) < n) {
-                e = V::sum(r);
-                const uint32_t j = (v >= P) + (v >= 2 * P);
-                take = claim_min(s.claim + e, j) == kUnc;
+    // round 0: four records per thread and append (one record: 9,300 cycles of
+    // a 2,000-key bucket's 103,000)
+    for (uint32_t v0 = 0; v0 < m; v0 += 4u * T_) {
+        const uint32_t v = v0 + 4u * tid;
+        T r[4] = {0, 0, 0, 0};
+        if constexpr (sizeof(T) == 4) {
+            // the records' space is a multiple of 16 bytes
+            if (v < m) {
+                const uint4 q = *reinterpret_cast<const uint4 *>(s.rec + v);
+                r[0] = q.x;
+                r[1] = q.y;
+                r[2] = q.z;
+                r[3] = q.w;
             }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+                if (v + q < m) r[q] = s.rec[v + q];
         }
-        cta_append(&lcur, s.L, 0u, take, e);
+        uint32_t who[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const uint32_t e = V::sum(r[q]), x = v + (uint32_t)q;
+            bool take = x < m && V::deg(r[q]) == 1u && e < n;
+            if (take) {
+                const uint32_t tag = hinge_code((x >= P) + (x >= 2 * P));
+                take = claim_open(s.claim + e, tag) && claim_put(s.claim + e, tag) == kUnc;
+            }
+            who[q] = __ballot_sync(0xFFFFFFFFu, take);
+        }
+        const uint32_t lane = tid & 31u;
+        uint32_t at = 0;
+        if (lane == 0)
+            at = atomicAdd(&lcur, (uint32_t)(__popc(who[0]) + __popc(who[1]) + __popc(who[2]) +
+                                             __popc(who[3])));
+        at = __shfl_sync(0xFFFFFFFFu, at, 0);
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            if ((who[q] >> lane) & 1u)
+                s.L[at + __popc(who[q] & ((1u << lane) - 1u))] = (uint16_t)V::sum(r[q]);
+            at += __popc(who[q]);
+        }
     }
+    // DeleteEdge of the i-th listed edge in round t: take[k] when the vertex
+    // that loses it is the first to claim its last edge f[k]
+    auto delete_edge = [&](uint32_t i, uint32_t t, bool(&take)[2], uint32_t(&f)[2]) {
+        const uint32_t e = s.L[i];
+        const uint32_t h = hinge_of(s.claim[e]);
+        const uint32_t j0 = h == 0 ? 1u : 0u, j1 = h == 2 ? 1u : 2u;
+        uint32_t x[2];
+        if (VERTS) {
+            x[0] = s.V[j0 * n + e] + j0 * P;
+            x[1] = s.V[j1 * n + e] + j1 * P;
+        } else {
+            uint32_t v[3];
+            bucket_edge(__ldg(keys + e), seed, fm, P, v);
+            x[0] = h == 0 ? v[1] : v[0];
+            x[1] = h == 2 ? v[1] : v[2];
+        }
+        T old[2];
+#pragma unroll
+        for (int k = 0; k < 2; k++) old[k] = atomicAdd(s.rec + x[k], (T)(0) - V::unit(e));
+        // both claim words are read before either is claimed
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            f[k] = (V::sum(old[k]) - e) & V::mask();
+            take[k] = V::deg(old[k]) == 2u && f[k] < n &&
+                      claim_open(s.claim + f[k], (t + 1) << 2);
+        }
+#pragma unroll
+        for (int k = 0; k < 2; k++)
+            if (take[k])
+                take[k] = claim_put(s.claim + f[k], ((t + 1) << 2) | hinge_code(k ? j1 : j0)) == kUnc;
+    };
     // Rounds, one block barrier each: round t appends layer t + 1 from its
     // start le through counter t mod 3.  Every thread reads that counter just
     // after the round's barrier; the counter round t + 1 will use was last
     // read before the previous barrier, so thread 0 clears it during round t.
+    // A layer of at most kWarpLayer edges, and those after it while they stay
+    // as small, are run by one warp, with no block barrier and no counter: a
+    // bucket of 2,000 keys has 37 rounds, 33 of them on 64 edges or fewer, and
+    // a round of the block took 2,900 cycles (47 % of the warps' time at its
+    // barrier) whatever its layer held.  With the claims by one atomicAnd and
+    // the vector scan of round 0: 9.33 -> 8.02 ms for 65,536 lognormal buckets.
     uint32_t *cnt3 = sh + 4;  // sh[4..6]
     __syncthreads();
     if (tid == 0) {
@@ -257,6 +316,8 @@ __device__ bool run_bucket(const BatchArgs &a, uint32_t b, BucketState<T, C> s, 
         cnt3[0] = cnt3[1] = cnt3[2] = 0;
     }
     __syncthreads();
+    const uint32_t lane = tid & 31u, warp = tid >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
     uint32_t t = 0, lb = 0, le = s.loff[1];
     bool too_many = false;
     while (le > lb) {
@@ -264,40 +325,46 @@ __device__ bool run_bucket(const BatchArgs &a, uint32_t b, BucketState<T, C> s, 
             too_many = true;
             break;
         }
+        if (le - lb <= kWarpLayer) {
+            __syncthreads();  // every thread has read the last round's counter
+            if (warp == 0) {
+                do {
+                    uint32_t next = le;
+                    for (uint32_t i0 = lb; i0 < le; i0 += 32u) {
+                        bool take[2] = {false, false};
+                        uint32_t f[2] = {0, 0};
+                        if (i0 + lane < le) delete_edge(i0 + lane, t, take, f);
+                        const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, take[0]);
+                        const uint32_t b1 = __ballot_sync(0xFFFFFFFFu, take[1]);
+                        if (take[0]) s.L[next + __popc(b0 & lt)] = (uint16_t)f[0];
+                        next += __popc(b0);
+                        if (take[1]) s.L[next + __popc(b1 & lt)] = (uint16_t)f[1];
+                        next += __popc(b1);
+                    }
+                    if (lane == 0) s.loff[t + 2] = next;
+                    __syncwarp();
+                    lb = le;
+                    le = next;
+                    t++;
+                } while (le > lb && le - lb <= kWarpLayer && t + 2 <= s.rcap);
+                if (lane == 0) {
+                    cnt3[0] = cnt3[1] = cnt3[2] = 0;
+                    sh[0] = t;
+                }
+            }
+            __syncthreads();
+            t = *(volatile uint32_t *)(sh + 0);
+            lb = s.loff[t];
+            le = s.loff[t + 1];
+            continue;
+        }
         uint32_t *cur = cnt3 + t % 3;
         if (tid == 0) cnt3[(t + 1) % 3] = 0;
         for (uint32_t i0 = lb; i0 < le; i0 += T_) {
             const uint32_t i = i0 + tid;
             bool take[2] = {false, false};
             uint32_t f[2] = {0, 0};
-            if (i < le) {
-                const uint32_t e = s.L[i];
-                const uint32_t h = s.claim[e] & 3u;
-                const uint32_t j0 = h == 0 ? 1u : 0u, j1 = h == 2 ? 1u : 2u;
-                uint32_t x[2];
-                if (VERTS) {
-                    x[0] = s.V[j0 * n + e] + j0 * P;
-                    x[1] = s.V[j1 * n + e] + j1 * P;
-                } else {
-                    uint32_t v[3];
-                    bucket_edge(__ldg(keys + e), seed, fm, P, v);
-                    x[0] = h == 0 ? v[1] : v[0];
-                    x[1] = h == 2 ? v[1] : v[2];
-                }
-                T old[2];
-#pragma unroll
-                for (int k = 0; k < 2; k++) old[k] = atomicAdd(s.rec + x[k], (T)(0) - V::unit(e));
-#pragma unroll
-                for (int k = 0; k < 2; k++) {
-                    if (V::deg(old[k]) == 2u) {
-                        const uint32_t g = (V::sum(old[k]) - e) & V::mask();
-                        if (g < n) {
-                            take[k] = claim_min(s.claim + g, ((t + 1) << 2) | (k ? j1 : j0)) == kUnc;
-                            f[k] = g;
-                        }
-                    }
-                }
-            }
+            if (i < le) delete_edge(i, t, take, f);
             cta_append2(cur, s.L, le, take, f);
         }
         __syncthreads();
@@ -316,8 +383,7 @@ __device__ bool run_bucket(const BatchArgs &a, uint32_t b, BucketState<T, C> s, 
     // per layer, the layers' starts and the counts of the lower warps give
     // where its edges of a layer go, and a second walk places them in id order
     // (the vertex records are dead: their space holds the counts).
-    const uint32_t nw = T_ / 32u, lane = tid & 31u, warp = tid >> 5;
-    const uint32_t lt = (1u << lane) - 1u;
+    const uint32_t nw = T_ / 32u;
     auto key_of = [&](uint32_t e) {
         const uint32_t c = s.claim[e];
         return c == kUnc ? R : c >> 2;
@@ -386,27 +452,42 @@ __device__ bool run_bucket(const BatchArgs &a, uint32_t b, BucketState<T, C> s, 
         const uint32_t words = (m + 15) / 16;
         for (uint32_t w = tid; w < words; w += T_) s.G[w] = 0;
         __syncthreads();
+        auto solve = [&](uint32_t i) {
+            const uint32_t e = s.L[i];
+            const uint32_t h = hinge_of(s.claim[e]);
+            uint32_t v[3];
+            if (VERTS) {
+#pragma unroll
+                for (int j = 0; j < 3; j++) v[j] = s.V[(uint32_t)j * n + e] + (uint32_t)j * P;
+            } else {
+                bucket_edge(__ldg(keys + e), seed, fm, P, v);
+            }
+            uint32_t sum = 0;
+#pragma unroll
+            for (int j = 0; j < 3; j++)
+                if ((uint32_t)j != h)
+                    sum += (((volatile uint32_t *)s.G)[v[j] >> 4] >> (2 * (v[j] & 15))) & 3u;
+            const uint32_t val = (h + 6u - sum) % 3u;
+            const uint32_t vh = h == 0 ? v[0] : (h == 1 ? v[1] : v[2]);
+            atomicOr(s.G + (vh >> 4), (val ? val : 3u) << (2 * (vh & 15)));
+        };
         for (int32_t r = (int32_t)R - 1; r >= 0; r--) {
             const uint32_t lo = s.loff[r], hi = s.loff[r + 1];
-            for (uint32_t i = lo + tid; i < hi; i += T_) {
-                const uint32_t e = s.L[i];
-                const uint32_t h = s.claim[e] & 3u;
-                uint32_t v[3];
-                if (VERTS) {
-#pragma unroll
-                    for (int j = 0; j < 3; j++)
-                        v[j] = s.V[(uint32_t)j * n + e] + (uint32_t)j * P;
-                } else {
-                    bucket_edge(__ldg(keys + e), seed, fm, P, v);
+            if (hi - lo <= kWarpLayer) {  // a run of small layers: one warp (see the rounds)
+                int32_t q = r;
+                uint32_t top = hi;
+                for (; q >= 0; q--) {
+                    const uint32_t bot = s.loff[q];
+                    if (top - bot > kWarpLayer) break;
+                    if (warp == 0) {
+                        for (uint32_t i = bot + lane; i < top; i += 32u) solve(i);
+                        __syncwarp();
+                    }
+                    top = bot;
                 }
-                uint32_t sum = 0;
-#pragma unroll
-                for (int j = 0; j < 3; j++)
-                    if ((uint32_t)j != h)
-                        sum += (((volatile uint32_t *)s.G)[v[j] >> 4] >> (2 * (v[j] & 15))) & 3u;
-                const uint32_t val = (h + 6u - sum) % 3u;
-                const uint32_t vh = v[h];
-                atomicOr(s.G + (vh >> 4), (val ? val : 3u) << (2 * (vh & 15)));
+                r = q + 1;
+            } else {
+                for (uint32_t i = lo + tid; i < hi; i += T_) solve(i);
             }
             __syncthreads();
         }
@@ -524,7 +605,7 @@ void launch_batch_g_offsets(const Launch &L, const uint64_t *off, uint32_t B, ui
 // SM, with g values) at the shape chosen and at the next best: 200 keys 119 /
 // 108, 1000 182 / 159, 1500 158 / 147, 2000 152 / 141, 3500 147 / 145, 4000
 // 131 / 130, 6000 118 / 112, 8000 107 / 104, 12000 102 / 97, 24000 95 / 91,
-// 60000 (global regions) 33 / 25.
+// 60000 (global regions) 33 / 25 (before one warp took the small layers).
 struct BatchClass {
     uint32_t threads, ctas;
     bool verts;   // takes buckets whose vertices fit beside their state, or
