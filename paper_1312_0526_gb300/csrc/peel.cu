@@ -591,7 +591,7 @@ void launch_round(const Launch &L, uint32_t r, bool gen, const RoundParams *prm,
 
 // ------------------------------------------------------------------ tails --
 // Rounds over small layers, one after the other in one launch of one cluster.
-// A launch of k_round costs 12 us however small its layer is (launch, while
+// A turn of the loop with one k_round costs 12 us however small its layer (launch, while
 // node, then eight dependent trips to L2: parameters, round, layer start,
 // entries, atomics, claims, list cursor, closing count), and a peel spends
 // most of its rounds on layers of a few thousand edges; close above the
