@@ -385,7 +385,7 @@ hpeel_status hpeel_mphf_build_async(const uint64_t *d_keys, uint64_t n, uint64_t
  * hashing, peel, hinges, g values and rank directory, bit for bit, for any n
  * both accept -- with 64-bit edge and vertex ids.  n may reach the size at
  * which a part of m / 3 vertices still has 32-bit local ids (about 1.05e10
- * keys at gamma = 1.23).  The state is compact: 8 bytes per vertex, 4 per
+ * keys at gamma = 1.23; n < 2^39 whatever gamma is).  The state is compact: 8 bytes per vertex, 4 per
  * key of claim words, 8 per key of layer list; no edge is stored (an edge's
  * vertices are hashed again from its key when needed), so the keys must stay
  * readable by the device during the call.  No canonical order output.
@@ -402,8 +402,8 @@ hpeel_status hpeel_mphf_build_async(const uint64_t *d_keys, uint64_t n, uint64_t
  *              bytes, 256-byte aligned.
  *   seed, gamma_milli, max_tries, h_stats: as hpeel_mphf_build (retries with
  *   seed + 1, ...; h_stats->seed_used is the seed lookups must use).
- * Synchronises stream.  Errors: HPEEL_ERR_INVALID_ARG (m / 3 >= 2^32, h_list
- * not page-locked), HPEEL_ERR_WORKSPACE_TOO_SMALL, HPEEL_ERR_RETRIES_EXHAUSTED,
+ * Synchronises stream.  Errors: HPEEL_ERR_INVALID_ARG (m / 3 >= 2^32, n >= 2^39,
+ * h_list not page-locked), HPEEL_ERR_WORKSPACE_TOO_SMALL, HPEEL_ERR_RETRIES_EXHAUSTED,
  * HPEEL_ERR_CAPACITY (more than HPEEL_MAX_ROUNDS rounds, or a vertex of degree
  * 2^24 or more), HPEEL_ERR_DEVICE_CHECK, HPEEL_ERR_CUDA.
  */

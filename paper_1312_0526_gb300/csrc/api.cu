@@ -2038,10 +2038,13 @@ hpeel_status hpeel_mphf_build_large(const uint64_t *d_keys, uint64_t n, uint64_t
     if (max_tries == 0) return fail(HPEEL_ERR_INVALID_ARG, "max_tries must be positive");
     const LargeLayout lay = large_layout(n, gamma_milli, h_list != nullptr);
     const uint64_t m = lay.m, P = m / 3;
-    if (P >= (1ull << 32) || n >= (1ull << 40))
+    if (P >= (1ull << 32))
         return fail(HPEEL_ERR_INVALID_ARG,
                     "n = %llu: a part of m / 3 vertices needs ids below 2^32",
                     (unsigned long long)n);
+    if (n >= (1ull << kLargeIdBits))
+        return fail(HPEEL_ERR_INVALID_ARG, "n = %llu: edge ids must be below 2^%d",
+                    (unsigned long long)n, kLargeIdBits);
     Launch L;
     HP_TRY(make_launch(stream, &L));
     if (n == 0) {

@@ -314,7 +314,9 @@ void launch_emit_advance(const Launch &L, EmitState *es, const uint32_t *loff, u
 void launch_layer_off_dev(const Launch &L, const uint32_t *loff, const Ctl *ctl,
                           uint32_t max_layers, uint64_t *out);
 
-// f4: MPHF build beyond 32-bit ids (large.cu).
+// f4: MPHF build beyond 32-bit ids (large.cu).  A vertex record keeps the sum of
+// its edges' ids modulo 2^kLargeIdBits, so ids stay below that.
+constexpr int kLargeIdBits = 39;
 RoundLaunch large_round_launch(const Launch &L, bool first);
 void launch_large_set_params(const Launch &L, LargeParams *dst, const LargeParams &v);
 // The build by vertex range: chunks of 2^kLargeChunk vertices of a part, per_pass

@@ -41,9 +41,9 @@ namespace hp {
 
 constexpr uint32_t kLDegBits = 24;
 constexpr unsigned long long kLDegMask = (1ull << kLDegBits) - 1ull;
-// ids below 2^39: the claim words alone of more edges would take 2 TB
-constexpr unsigned long long kLSumMask = (1ull << 39) - 1ull;
-constexpr unsigned long long kLMark = 1ull << 63;
+constexpr unsigned long long kLSumMask = (1ull << kLargeIdBits) - 1ull;
+constexpr unsigned long long kLMark = 1ull << (kLDegBits + kLargeIdBits);
+static_assert(kLDegBits + kLargeIdBits == 63, "degree, id sum and mark fill a record");
 constexpr int kLPosShift = 62;
 constexpr unsigned long long kLIdMask = (1ull << kLPosShift) - 1ull;
 
@@ -437,8 +437,9 @@ LargeBuildPlan large_build_plan(uint64_t n, uint64_t P, uint64_t room) {
     const uint64_t head = ((uint64_t)b.chunks * 8 + 255) & ~255ull;
     const uint64_t fit = room > head ? (room - head) / (8 * b.cap) : 0;
     b.per_pass = (uint32_t)std::min<uint64_t>(b.chunks, std::min<uint64_t>(fit, 2048));
-    // ids of 40 bits; a few passes over the keys per part at most
-    if (n >= (1ull << 40) || b.per_pass == 0 || (b.chunks + b.per_pass - 1) / b.per_pass > 4)
+    // a few passes over the keys per part at most
+    static_assert(kLargeIdBits <= 40 && kLargeChunk <= 24, "a pair is {vertex : 24, edge id : 40}");
+    if (b.per_pass == 0 || (b.chunks + b.per_pass - 1) / b.per_pass > 4)
         b.per_pass = 0;
     return b;
 }
