@@ -73,9 +73,11 @@ typedef struct hpeel_stats {
     uint64_t hinge_moves;   /* peeled edges whose first claim came from a
                                vertex other than the hinge (a vertex of
                                smaller position claimed later in the round);
-                               0 where a round's claims are all in before its
-                               layer is listed: sorted rounds, and graphs of
-                               up to about 131,000 edges peeled in one launch */
+                               0 in sorted rounds, whose claims are all in
+                               before their layer is listed; graphs of up to
+                               about 131,000 edges peeled in one launch, whose
+                               rounds have no first claim, count every edge
+                               that two or more vertices claim in its round */
     uint32_t async_status;  /* the *_async calls: 1 done (outputs written),
                                2 no seed peeled (builds), 3 device check
                                failed (device_err holds the code), 4 more

@@ -1321,6 +1321,7 @@ hpeel_status peel_entry(bool general, const uint32_t *d_edges, uint64_t n, uint6
             h_stats->core_nonempty = ps->core_nonempty;
             h_stats->first_layer = ps->first_layer;
             h_stats->frontier = ps->frontier;
+            h_stats->hinge_moves = ps->hinge_moves;
         }
         return HPEEL_OK;
     }

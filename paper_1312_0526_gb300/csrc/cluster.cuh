@@ -73,6 +73,18 @@ __device__ __forceinline__ void cl_red_or(uint32_t a, uint32_t v) {
                      : "memory");
 }
 template <bool SOLO>
+__device__ __forceinline__ uint32_t cl_min(uint32_t a, uint32_t v) {
+    uint32_t old;
+    if (SOLO)
+        asm volatile("atom.relaxed.cta.shared::cta.min.u32 %0, [%1], %2;"
+                     : "=r"(old) : "r"(a), "r"(v) : "memory");
+    else
+        asm volatile("atom.relaxed.cluster.shared::cluster.min.u32 %0, [%1], %2;"
+                     : "=r"(old) : "r"(a), "r"(v) : "memory");
+    return old;
+}
+
+template <bool SOLO>
 __device__ __forceinline__ void cl_red_min(uint32_t a, uint32_t v) {
     if (SOLO)
         asm volatile("red.relaxed.cta.shared::cta.min.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");

@@ -23,8 +23,8 @@
 //
 // Rounds.  Layer t is the set of edges whose claim word holds round t.  There
 // is no layer list: the atomic that takes a vertex from degree 2 to 1 names
-// its last edge f (old sum - e), and the vertex's claim is a fire-and-forget
-// minimum on f's claim word in its owner's shared memory; the owner finds its
+// its last edge f (old sum - e), and the vertex's claim is a minimum on f's claim
+// word in its owner's shared memory that nothing waits for; the owner finds its
 // part of the next layer in its own claim words.  All claims of a round are
 // in before the barrier, so the claim word names the hinge when the edge is
 // deleted.  Three forms, by size:
@@ -67,6 +67,7 @@ struct SmallShared {
     uint32_t deg;      // sum of the degrees of this block's vertices
     uint32_t bad;      // an input edge of this block is invalid
     uint32_t cross;    // vertices that fell from degree 2 to 1
+    uint32_t moves;    // this block's edges with two claims or more in their round
     uint32_t err;      // device error code of this block
     uint32_t peeled;   // peeled edges of this block
     uint32_t first;    // those of layer 0
@@ -95,10 +96,11 @@ struct SmallView {
     uint32_t e0, ne;            // first edge and edges of this block
     uint32_t vslots;            // vertex slots of a block
     uint32_t *claim, *rec;      // [epc], [vslots]
+    uint32_t *hits;             // claims of this block's edges beyond the first (small_claim)
     uint32_t *bits;             // EPT = 16: [2][epc / 32], claims of even and odd rounds
     uint16_t *list;             // EPT = 16: [epc] this block's edges in the order they go
     V *vert;                    // [R][epc] (EPT = 16, or a general graph)
-    uint32_t s_claim, s_rec, s_bits, s_vert;
+    uint32_t s_claim, s_rec, s_hits, s_bits, s_vert;
 };
 
 template <bool SOLO>
@@ -124,11 +126,26 @@ __device__ __forceinline__ uint32_t edge_vertex(const SmallArgs &a, const SmallV
     return (uint32_t)w.vert[j * a.epc + i] + (GEN ? 0u : j * a.P);
 }
 
+// A cluster's claims of one thread for one round, whose outcomes have not been
+// looked at: the claim words they found (all ones: none, or the edge's first
+// claim) and their edges.
+template <int N>
+struct SmallPending {
+    uint32_t old[N], edge[N], t;
+};
+
 // Claim of edge f for round t by vertex x at position j of
 // its edges (in a general graph: at the first slot of f's row that holds x).
+// Edges with two claims or more are counted.  In one block each edge has a byte,
+// 4 bits for the claims of even rounds and 4 for those of odd ones: an edge
+// deleted in round t has claims for t, and late ones for t + 1, which do not
+// count (one more local addition; looking at the minimum's result takes 1 us
+// more of 12.6 for a peel of 1009 edges).  In a cluster a second remote atomic
+// takes 8 us more of 148 for a peel of 1e5 edges, the minimum's result (`old`),
+// looked at later, 3.
 template <int R, bool GEN, bool SOLO, bool BITS>
 __device__ __forceinline__ void small_claim(const SmallArgs &a, const SmallView<GEN> &w, uint32_t f,
-                                            uint32_t x, uint32_t j, uint32_t t) {
+                                            uint32_t x, uint32_t j, uint32_t t, uint32_t &old) {
     const uint32_t o = edge_owner<SOLO>(a, f), i = f - o * a.epc;
     if (GEN) {
         j = R - 1;
@@ -138,10 +155,37 @@ __device__ __forceinline__ void small_claim(const SmallArgs &a, const SmallView<
                     ? (uint32_t)k
                     : j;
     }
-    cl_red_min<SOLO>(cl_map<SOLO>(w.s_claim + 4u * i, o), (t << 2) | j);
+    const uint32_t at = cl_map<SOLO>(w.s_claim + 4u * i, o);
+    if (SOLO) {
+        cl_red_min<SOLO>(at, (t << 2) | j);
+        cl_red_add<SOLO>(w.s_hits + (i & ~3u), 1u << (8u * (i & 3u) + 4u * (t & 1u)));
+    } else {
+        old = cl_min<SOLO>(at, (t << 2) | j);
+    }
     if (BITS && t >= kSmScan)
         cl_red_or<SOLO>(cl_map<SOLO>(w.s_bits + 4u * ((t & 1u) * (a.epc >> 5) + (i >> 5)), o),
                         1u << (i & 31u));
+}
+
+// Looks at a thread's last claims: an edge that had a claim for the same round gets
+// its bit in its owner's `hits`.  The order does not matter, so this is done
+// while the thread waits for the vertices of the next edge it deletes, and
+// nothing in it is waited for.
+template <bool GEN, int N>
+__device__ __forceinline__ void small_settle(const SmallArgs &a, const SmallView<GEN> &w,
+                                             SmallPending<N> &p) {
+    uint32_t all = kUnclaimed;
+#pragma unroll
+    for (int q = 0; q < N; q++) all &= p.old[q];
+    if (all == kUnclaimed) return;
+#pragma unroll
+    for (int q = 0; q < N; q++) {
+        if ((p.old[q] >> 2) == p.t) {
+            const uint32_t o = edge_owner<false>(a, p.edge[q]), i = p.edge[q] - o * a.epc;
+            cl_red_or<false>(cl_map<false>(w.s_hits + 4u * (i >> 5), o), 1u << (i & 31u));
+        }
+        p.old[q] = kUnclaimed;
+    }
 }
 
 struct SmallPeel {
@@ -170,12 +214,14 @@ __device__ __forceinline__ bool small_edge(const SmallArgs &a, uint64_t seed, ui
 
 // DeleteEdge of edge e with hinge position h in round t: its other vertices
 // lose it, and one that falls to degree 1 claims its last edge for round t + 1.
+// pend: a cluster thread's last claims, then those made here.
 // at(q): record address of the q-th vertex that is not the hinge, id(q) its id
 // (called for WIDE and general graphs only).
 template <int R, bool GEN, bool SOLO, bool BITS, bool WIDE, typename At, typename Id>
 __device__ __forceinline__ void small_delete(const SmallArgs &a, const SmallView<GEN> &w,
                                              SmallShared &sh, uint32_t e, uint32_t h, uint32_t t,
-                                             At at, Id id, uint32_t &cross) {
+                                             At at, Id id, uint32_t &cross,
+                                             SmallPending<R - 1> &pend) {
     uint32_t deg[R - 1], f[R - 1];
 #pragma unroll
     for (int q = 0; q < R - 1; q++) {
@@ -188,6 +234,10 @@ __device__ __forceinline__ void small_delete(const SmallArgs &a, const SmallView
             deg[q] = cl_add<SOLO>(at(q), 0u - ((e << kSmDegBits) + 1u));
         }
     }
+    if (!SOLO) {
+        small_settle(a, w, pend);
+        pend.t = t + 1u;
+    }
     if (!WIDE) {
 #pragma unroll
         for (int q = 0; q < R - 1; q++) {
@@ -199,18 +249,21 @@ __device__ __forceinline__ void small_delete(const SmallArgs &a, const SmallView
     for (int q = 0; q < R - 1; q++) {
         if (deg[q] != 2u) continue;
         cross++;
-        if (f[q] < a.n)
+        if (f[q] < a.n) {
             small_claim<R, GEN, SOLO, BITS>(a, w, f[q], GEN ? id(q) : 0u,
-                                            (uint32_t)q + ((uint32_t)q >= h ? 1u : 0u), t + 1u);
-        else
+                                            (uint32_t)q + ((uint32_t)q >= h ? 1u : 0u), t + 1u,
+                                            pend.old[q]);
+            pend.edge[q] = f[q];
+        } else {
             sh.err = kDevBadEdge;
+        }
     }
 }
 // The same for this block's edge i, from its stored vertices.
 template <int R, bool GEN, bool SOLO, bool WIDE>
 __device__ __forceinline__ void small_delete_at(const SmallArgs &a, const SmallView<GEN> &w,
                                                 SmallShared &sh, uint32_t i, uint32_t t,
-                                                uint32_t &cross) {
+                                                uint32_t &cross, SmallPending<R - 1> &pend) {
     const uint32_t h = w.claim[i] & 3u;
     uint32_t x[R - 1];
 #pragma unroll
@@ -218,7 +271,7 @@ __device__ __forceinline__ void small_delete_at(const SmallArgs &a, const SmallV
         x[q] = edge_vertex(a, w, i, (uint32_t)q + ((uint32_t)q >= h ? 1u : 0u));
     small_delete<R, GEN, SOLO, true, WIDE>(
         a, w, sh, w.e0 + i, h, t, [&](int q) { return rec_addr<SOLO>(w, x[q]); },
-        [&](int q) { return x[q]; }, cross);
+        [&](int q) { return x[q]; }, cross, pend);
 }
 
 // One peel: records, round 0 and the rounds.  Every thread of the cluster
@@ -240,10 +293,12 @@ __device__ uint32_t small_peel(const SmallArgs &a, const SmallView<GEN> &w, Smal
         if (WIDE && slot_vertex(w, i) < m) a.wide[slot_vertex(w, i)] = 0ull;
     }
     for (uint32_t i = tid; i < a.epc; i += T) w.claim[i] = kUnclaimed;
+    for (uint32_t i = tid; i < (SOLO ? a.epc >> 2 : a.epc >> 5); i += T) w.hits[i] = 0;
     if (BITS)
         for (uint32_t i = tid; i < (a.epc >> 4); i += T) w.bits[i] = 0;
     if (tid < 4) sh.any[tid] = sh.all[tid] = 0;
-    if (tid == 4) sh.deg = sh.bad = sh.cross = sh.err = sh.peeled = sh.first = sh.listed = 0;
+    if (tid == 4)
+        sh.deg = sh.bad = sh.cross = sh.moves = sh.err = sh.peeled = sh.first = sh.listed = 0;
     cl_sync<SOLO>();
     // AddEdge of this block's edges, four keys in flight per thread
     constexpr int kU = BITS ? 4 : EPT;
@@ -285,22 +340,34 @@ __device__ uint32_t small_peel(const SmallArgs &a, const SmallView<GEN> &w, Smal
     cl_sync<SOLO>();
     // round 0: every vertex of degree 1 claims its edge
     {
+        constexpr int kV = SOLO ? 1 : 4;  // a cluster's claims in flight per thread
         uint32_t degs = 0;
-        for (uint32_t i = tid; i < w.vslots; i += T) {
-            const uint32_t v = slot_vertex(w, i);
-            uint32_t deg, f;
-            if (WIDE) {
-                const unsigned long long r = v < m ? __ldcg(a.wide + v) : 0ull;
-                deg = (uint32_t)r;
-                f = (uint32_t)(r >> 32);
-            } else {
-                const uint32_t r = w.rec[i];
-                deg = r & kSmDegMask;
-                f = r >> kSmDegBits;
+        for (uint32_t i0 = tid; i0 < w.vslots; i0 += kV * T) {
+            SmallPending<kV> pend;
+            pend.t = 0;
+#pragma unroll
+            for (int u = 0; u < kV; u++) {
+                pend.old[u] = kUnclaimed;
+                const uint32_t i = i0 + (uint32_t)u * T;
+                if (i >= w.vslots) continue;
+                const uint32_t v = slot_vertex(w, i);
+                uint32_t deg, f;
+                if (WIDE) {
+                    const unsigned long long r = v < m ? __ldcg(a.wide + v) : 0ull;
+                    deg = (uint32_t)r;
+                    f = (uint32_t)(r >> 32);
+                } else {
+                    const uint32_t r = w.rec[i];
+                    deg = r & kSmDegMask;
+                    f = r >> kSmDegBits;
+                }
+                degs += deg;
+                pend.edge[u] = f;
+                if (deg == 1u && f < n)
+                    small_claim<R, GEN, SOLO, BITS>(a, w, f, v, GEN ? 0u : part_of<R>(v, a.P), 0u,
+                                                    pend.old[u]);
             }
-            degs += deg;
-            if (deg == 1u && f < n)
-                small_claim<R, GEN, SOLO, BITS>(a, w, f, v, GEN ? 0u : part_of<R>(v, a.P), 0u);
+            if (!SOLO) small_settle(a, w, pend);
         }
         if (BITS && !WIDE) {  // EPT < 16: at most 4096 edges, no degree can overflow
             degs = __reduce_add_sync(0xFFFFFFFFu, degs);
@@ -319,6 +386,13 @@ __device__ uint32_t small_peel(const SmallArgs &a, const SmallView<GEN> &w, Smal
             return kDevCapacity;
     }
     uint32_t cross = 0, t = 0;
+    SmallPending<R - 1> pend;
+    pend.t = 0;
+#pragma unroll
+    for (int q = 0; q < R - 1; q++) {
+        pend.old[q] = kUnclaimed;
+        pend.edge[q] = 0;
+    }
     if constexpr (!BITS) {
         for (;; t++) {
             uint32_t c[EPT];
@@ -338,7 +412,7 @@ __device__ uint32_t small_peel(const SmallArgs &a, const SmallView<GEN> &w, Smal
                 auto at = [&](int q) { return (uint32_t)q >= h ? addr[k][q + 1] : addr[k][q]; };
                 small_delete<R, GEN, SOLO, BITS, WIDE>(
                     a, w, sh, tid * EPT + (uint32_t)k, h, t, at,
-                    [&](int q) { return (at(q) - w.s_rec) >> 2; }, cross);
+                    [&](int q) { return (at(q) - w.s_rec) >> 2; }, cross, pend);
             }
             if (!__syncthreads_or(hit)) break;
         }
@@ -393,7 +467,7 @@ __device__ uint32_t small_peel(const SmallArgs &a, const SmallView<GEN> &w, Smal
                 const uint32_t i = 16u * tid + __ffs(mask) - 1u;
                 uint32_t base = 0;
                 if (LIST && lane == 0) base = atomicAdd(&sh.listed, __popc(who));
-                if (mask) small_delete_at<R, GEN, SOLO, WIDE>(a, w, sh, i, t, cross);
+                if (mask) small_delete_at<R, GEN, SOLO, WIDE>(a, w, sh, i, t, cross, pend);
                 if (LIST) {
                     base = __shfl_sync(0xFFFFFFFFu, base, 0);
                     if (mask) w.list[base + __popc(who & ((1u << lane) - 1u))] = (uint16_t)i;
@@ -413,7 +487,7 @@ __device__ uint32_t small_peel(const SmallArgs &a, const SmallView<GEN> &w, Smal
                     w.list[at] = (uint16_t)(16u * tid + __ffs(mask) - 1u);
                 __syncwarp();
                 for (uint32_t k = lane; k < total; k += 32u)
-                    small_delete_at<R, GEN, SOLO, WIDE>(a, w, sh, w.list[base + k], t, cross);
+                    small_delete_at<R, GEN, SOLO, WIDE>(a, w, sh, w.list[base + k], t, cross, pend);
             }
             if (SOLO) {
                 if (!__syncthreads_or(hit)) break;
@@ -424,10 +498,14 @@ __device__ uint32_t small_peel(const SmallArgs &a, const SmallView<GEN> &w, Smal
         }
     }
     out.rounds = SOLO ? t : t - 2u;
+    if (!SOLO) small_settle(a, w, pend);
     // what was peeled: counted off the claim words
-    uint32_t peeled = 0, first = 0;
+    uint32_t peeled = 0, first = 0, moves = 0;
     for (uint32_t i = tid; i < w.ne; i += T) {
         const uint32_t c = w.claim[i];
+        // (an edge that is not peeled has no claims)
+        if (SOLO)
+            moves += ((reinterpret_cast<const uint8_t *>(w.hits)[i] >> (c & 4u)) & 15u) > 1u ? 1u : 0u;
         peeled += c != kUnclaimed ? 1u : 0u;
         first += c < 4u ? 1u : 0u;
     }
@@ -445,6 +523,11 @@ __device__ uint32_t small_peel(const SmallArgs &a, const SmallView<GEN> &w, Smal
         peeled = cl_load<SOLO>(cl_map<SOLO>(smem_u32(&sh.peeled), lane));
         first = cl_load<SOLO>(cl_map<SOLO>(smem_u32(&sh.first), lane));
     }
+    // (added to sh.moves, which is read after other barriers)
+    if (!SOLO)
+        for (uint32_t i = tid; i < (a.epc >> 5); i += T) moves += __popc(w.hits[i]);
+    moves = __reduce_add_sync(0xFFFFFFFFu, moves);
+    if (lane == 0 && moves) atomicAdd(&sh.moves, moves);
     out.peeled = __reduce_add_sync(0xFFFFFFFFu, peeled);
     out.first_layer = __reduce_add_sync(0xFFFFFFFFu, first);
     return 0u;
@@ -713,9 +796,11 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const SmallArgs a) {
     w.vslots = a.vslots;
     w.claim = small_smem;
     w.rec = w.claim + a.epc;
-    w.bits = w.rec + a.vslots;
+    w.hits = w.rec + a.vslots;
+    w.bits = w.hits + (SOLO ? a.epc >> 2 : a.epc >> 5);
     w.list = reinterpret_cast<uint16_t *>(w.bits + (EPT == 16 ? a.epc >> 4 : 0u));
     w.vert = reinterpret_cast<typename SmallView<GEN>::V *>(w.list + (EPT == 16 ? a.epc : 0u));
+    w.s_hits = smem_u32(w.hits);
     w.s_bits = smem_u32(w.bits);
     w.s_claim = smem_u32(w.claim);
     w.s_rec = smem_u32(w.rec);
@@ -750,12 +835,14 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const SmallArgs a) {
     }
     cl_sync<SOLO>();
     if (w.rank == 0 && threadIdx.x < 32u) {
-        uint32_t cross = 0, err = 0;
+        uint32_t cross = 0, moves = 0, err = 0;
         if (threadIdx.x < w.blocks) {
             cross = cl_load<SOLO>(cl_map<SOLO>(smem_u32(&sh.cross), threadIdx.x));
+            moves = cl_load<SOLO>(cl_map<SOLO>(smem_u32(&sh.moves), threadIdx.x));
             err = cl_load<SOLO>(cl_map<SOLO>(smem_u32(&sh.err), threadIdx.x));
         }
         cross = __reduce_add_sync(0xFFFFFFFFu, cross);
+        moves = __reduce_add_sync(0xFFFFFFFFu, moves);
         err = code ? code : __reduce_max_sync(0xFFFFFFFFu, err);
         if (threadIdx.x == 0) {
             hpeel_stats st{};
@@ -765,6 +852,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(const SmallArgs a) {
             st.device_err = err;
             st.first_layer = pe.first_layer;
             st.frontier = cross;
+            st.hinge_moves = moves;
             if (MODE == 0) {
                 st.core_nonempty = pe.peeled < a.n ? 1u : 0u;
                 st.async_status = err ? 3u : (a.layer_off && pe.rounds > a.max_layers ? 4u : 1u);
@@ -822,7 +910,7 @@ SmallShape small_shape(uint32_t n, uint32_t m, uint32_t r, bool gen, uint32_t bl
     // a cluster has one more warp for the bookkeeping
     const uint32_t want = ((s.epc / s.ept + 31u) & ~31u) + (blocks > 1 ? 32u : 0u);
     s.threads = want > kSmThreads ? kSmThreads : (want < 128u ? 128u : want);
-    size_t graph = 4 * ((size_t)s.epc + s.vslots);
+    size_t graph = 4 * ((size_t)s.epc + s.vslots) + (blocks > 1 ? s.epc / 8 : s.epc);
     if (s.ept == 16) graph += s.epc / 4 + 2 * (size_t)s.epc;
     if (s.ept == 16 || gen) graph += (gen ? 4 : 2) * (size_t)s.epc * r;
     const size_t order = 4 * ((size_t)s.epc + kSmBins * (3 + s.threads / 32u));
