@@ -131,6 +131,7 @@ struct BatchArgs {
     uint32_t smem_bytes;      // dynamic shared memory per CTA
     uint32_t smem_rounds;     // layer-table entries of a bucket in shared memory
     uint32_t global16_rounds; // layer-table entries on the 32-bit global path
+    uint32_t wait;            // 1: reads what the launch before it wrote
 };
 
 __host__ __device__ inline size_t a16(size_t x) { return (x + 15) & ~(size_t)15; }
@@ -514,6 +515,7 @@ __global__ void __launch_bounds__(1024, 2) k_batched(BatchArgs a) {
     extern __shared__ __align__(16) char smem[];
     __shared__ __align__(16) uint32_t sh[8];  // sh[2..3] hold a 64-bit value
     __shared__ uint32_t s_b;
+    if (a.wait) asm volatile("griddepcontrol.wait;" ::: "memory");
     // the next class's blocks may start as this one's leave (see launch_batched)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     char *region = a.scratch + (size_t)blockIdx.x * a.scratch_bytes;
@@ -521,7 +523,7 @@ __global__ void __launch_bounds__(1024, 2) k_batched(BatchArgs a) {
     for (;;) {
         if (threadIdx.x == 0) {
             const uint32_t k = lo < hi ? lo + atomicAdd(a.next, 1u) : hi;
-            s_b = k < hi ? a.sched[k] : 0xFFFFFFFFu;
+            s_b = k < hi ? __ldcg(a.sched + k) : 0xFFFFFFFFu;
         }
         __syncthreads();
         const uint32_t b = s_b;
@@ -647,6 +649,7 @@ k_batch_schedule(const uint64_t *off, uint32_t B, BatchShapes shapes, uint32_t p
                  uint32_t *ctl) {
     __shared__ uint32_t cnt[kBatchBins], total[kBatchBins], low[kBatchBins];
     const uint32_t tid = threadIdx.x, rank = cl_rank(), blocks = gridDim.x;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     auto bin_of = [&](uint32_t b) {
         const uint64_t n64 = off[b + 1] - off[b];
         const uint32_t n = (uint32_t)(n64 < 131071u ? n64 : 131071u);
@@ -710,6 +713,16 @@ void launch_batched(const Launch &L, const uint64_t *keys, const uint64_t *off, 
                     uint32_t smem_per_sm, uint32_t *sched, uint32_t *ctl, uint32_t *late,
                     char *scratch) {
     const bool classes = smem_per_sm != 0;
+    // Few buckets: a class with more blocks per SM than hold them all at once is
+    // left out (its buckets run in the next larger one), and no launch has more
+    // blocks than there are buckets.  An empty launch of a full grid costs
+    // 4 us, of few blocks 1.6.  Per call, buckets of one size; one launch of the
+    // default shape / all classes on full grids / this: 1 bucket of 64 keys
+    // 23 / 54 / 20 us, of 2,000 66 / 66 / 32, 16 of 64 28 / 54 / 22, 256 of 64
+    // 36 / 62 / 35, 256 of 2,000 154 / 100 / 75, 1,024 of 64 65 / 67 / 51.
+    uint32_t most = 0;
+    for (int c = kBatchClasses - 1; c >= 0; c--)
+        if (most == 0 || (uint64_t)L.sms * most < B) most = std::max(most, kBatchClass[c].ctas);
     BatchShapes sh{};
     sh.smem_rounds = smem_rounds;
     sh.gamma_milli = gamma_milli;
@@ -719,8 +732,9 @@ void launch_batched(const Launch &L, const uint64_t *keys, const uint64_t *off, 
     for (int c = 0; c < kBatchClasses; c++) {
         sh.launch[c] = (uint32_t)kBatchClass[c].launch;
         sh.verts[c] = kBatchClass[c].verts;
-        sh.smem[c] = classes ? std::min(smem_bytes, (smem_per_sm / kBatchClass[c].ctas - 1024 - 64) & ~15u)
-                             : 0u;
+        sh.smem[c] = classes && kBatchClass[c].ctas <= most
+                         ? std::min(smem_bytes, (smem_per_sm / kBatchClass[c].ctas - 1024 - 64) & ~15u)
+                         : 0u;
     }
     {
         uint32_t plain = classes ? 0u : 1u;
@@ -734,7 +748,7 @@ void launch_batched(const Launch &L, const uint64_t *keys, const uint64_t *off, 
     }
     BatchArgs a{keys, off, B, gamma_milli, sched, nullptr, ctl + kBatchCtlNext, nullptr, nullptr,
                 order, rounds, status, G, G_off, scratch, batched_scratch_bytes(gamma_milli),
-                smem_bytes, smem_rounds, global16_rounds};
+                smem_bytes, smem_rounds, global16_rounds, 0u};
     if (!classes) {
         count_launch();
         k_batched<<<ctas, threads, smem_bytes, L.stream>>>(a);
@@ -743,19 +757,21 @@ void launch_batched(const Launch &L, const uint64_t *keys, const uint64_t *off, 
     // The launches overlap: each lets the next one's blocks start as its own
     // leave (programmatic dependent launch; they share nothing but the
     // outputs, bucket by bucket), and ends only after the one before it.  The
+    // first waits for the schedule before it lets any other start.  The
     // last takes the buckets that needed more rounds than their class's shared
-    // memory holds; it shares the global regions with the first, so it starts
-    // when all others have ended.
+    // memory holds; it shares the global regions with the first, so it waits
+    // until all others have ended.
     for (int l = 0; l <= kBatchLaunches; l++) {
         const bool global = l == 0 || l == kBatchLaunches;
         BatchArgs x = a;
-        uint32_t th = 1024, per = 2;
+        uint32_t th = 1024, per = global ? 2 : 0;
         for (int c = 0; c < kBatchClasses && !global; c++)
-            if (kBatchClass[c].launch == l) {
+            if (kBatchClass[c].launch == l && sh.smem[c]) {
                 th = kBatchClass[c].threads;
                 per = kBatchClass[c].ctas;
                 x.smem_bytes = sh.smem[c];
             }
+        if (per == 0) continue;
         if (l < kBatchLaunches) {
             x.range = ctl + l;
             x.next = ctl + kBatchCtlNext + l;
@@ -764,6 +780,7 @@ void launch_batched(const Launch &L, const uint64_t *keys, const uint64_t *off, 
             x.range = ctl + kBatchCtlLate - 1;  // 0, the late buckets' count
             x.next = ctl + kBatchCtlLate + 1;
         }
+        x.wait = global ? 1u : 0u;
         if (global) {
             x.smem_bytes = 0;
         } else {
@@ -771,7 +788,7 @@ void launch_batched(const Launch &L, const uint64_t *keys, const uint64_t *off, 
             x.late_count = ctl + kBatchCtlLate;
         }
         cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3((unsigned)L.sms * per);
+        cfg.gridDim = dim3(std::min((unsigned)L.sms * per, B));
         cfg.blockDim = dim3(th);
         cfg.dynamicSmemBytes = x.smem_bytes;
         cfg.stream = L.stream;
@@ -779,7 +796,7 @@ void launch_batched(const Launch &L, const uint64_t *keys, const uint64_t *off, 
         at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at.val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = &at;
-        cfg.numAttrs = l > 0 && l < kBatchLaunches ? 1 : 0;
+        cfg.numAttrs = 1;
         void *args[] = {(void *)&x};
         count_launch();
         cudaLaunchKernelExC(&cfg, (const void *)k_batched, args);
