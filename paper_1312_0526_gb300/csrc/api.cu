@@ -390,11 +390,6 @@ hpeel_status launch_cached_graph(const Launch &L, const std::string &key, F capt
     return HPEEL_OK;
 }
 
-// Round kernels in one turn of the loop over large layers: a turn of a while
-// node costs about 3 us, a round kernel without a layer about as much, once
-// (general peel of 2e7 edges: 3.85 ms with one, 3.64 with four, 3.60 with eight).
-constexpr int kBodyRounds = 8;
-
 // Round 0 and the loops of rounds, added at the capture position of s0; the
 // loop bodies are captured on s1, a loop inside a loop on s2.  With a sorted
 // plan: round 0 and the first rounds in sorted form (a while node over sorted
@@ -484,11 +479,11 @@ cudaError_t capture_rounds(cudaStream_t s0, cudaStream_t s1, cudaStream_t s2, in
 }
 
 // Kernels one peel's rounds launched, from its control block: round 0 (6 in
-// sorted form), 7 per sorted round, 1 per random round, 2 per run of small
-// layers.
-uint64_t round_kernels(const Ctl &c, bool sorted) {
+// sorted form), 7 per sorted round, and those of the loop of random rounds,
+// which k_tail counts; without it 1 per random round.
+uint64_t round_kernels(const Ctl &c, bool sorted, bool tail) {
     const uint64_t rounds = (uint64_t)c.round + (c.more ? 1 : 0);
-    return (sorted ? 6 : 1) + 7ull * c.brounds + (rounds - c.brounds - c.trounds) + 2ull * c.tails;
+    return (sorted ? 6 : 1) + 7ull * c.brounds + (tail ? c.kernels : rounds - c.brounds);
 }
 
 // The device-driven round loop of a host-driven peel: round 0 and the loops
@@ -653,7 +648,7 @@ hpeel_status peel_core_rb(const Launch &L, const PeelIO &io, uint32_t n, uint32_
                                     cudaMemcpyDeviceToHost, L.stream));
         }
         HP_TRY(read_ctl());
-        count_launch((uint32_t)round_kernels(*hctl, sorted));
+        count_launch((uint32_t)round_kernels(*hctl, sorted, tail.tail_max != 0));
     }
     if (hctl->err == kDevRoundOverflow && sorted) {
         // a sorted round's buckets or claim list were full (a skewed input):

@@ -38,8 +38,8 @@ struct alignas(16) Ctl {
     uint32_t bmode;      // 1: the next round runs in sorted (bucketed) form
     uint32_t brounds;    // rounds run in sorted form
     uint32_t cvalid;     // 1: the incidence build left round 0's claims in the claim list
-    uint32_t tails;      // launches of the cluster kernel that runs small layers
-    uint32_t trounds;    // rounds it ran
+    uint32_t gate;       // round at the start of the turn of the loop of random rounds
+    uint32_t kernels;    // kernels that loop has launched (graphs with a k_tail)
     uint32_t pad[3];
 };
 

@@ -643,12 +643,18 @@ k_tail(const RoundParams *__restrict__ prm, cudaGraphConditionalHandle cond) {
     // nothing to do, or a state the loop around cannot leave behind: stop it
     // (the same decision in every block)
     const bool bad = more && (lb >= le || le > n || le - lb > tail_max);
+    // this turn's launches: the gate, whole bodies of round kernels for the
+    // layers that were too large, this kernel
+    auto count_turn = [&]() {
+        ctl->kernels += 2 + (t0 - ctl->gate + kBodyRounds - 1) / kBodyRounds * kBodyRounds;
+    };
     if (!more || bad) {
         if (rank == 0 && tid == 0) {
             if (bad) {
                 raise_err(ctl, kDevCapacity);
                 ctl->more = 0;
             }
+            count_turn();
             if (cond) cudaGraphSetConditional(cond, 0u);
         }
         return;
@@ -827,15 +833,15 @@ k_tail(const RoundParams *__restrict__ prm, cudaGraphConditionalHandle cond) {
         *reinterpret_cast<uint4 *>(&ctl->round) = make_uint4(t, lb, le, more);
         ctl->lcur = le;
         ctl->next_size = le - lb;
-        ctl->tails++;
-        ctl->trounds += t - t0;
+        count_turn();
         if (cond) cudaGraphSetConditional(cond, more);
     }
 }
 
 // h = the next layer is too large for k_tail.
 __global__ void k_tail_gate(const RoundParams *prm, cudaGraphConditionalHandle h) {
-    const Ctl *ctl = prm->ctl;
+    Ctl *ctl = prm->ctl;
+    ctl->gate = ctl->round;
     cudaGraphSetConditional(
         h, ctl->more && ctl->err == 0u && ctl->next_size > prm->tail_max ? 1u : 0u);
 }
