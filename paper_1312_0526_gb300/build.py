@@ -44,6 +44,7 @@ def _measure_sources():
 
 def _deps():
     return (_sources() + _measure_sources() + glob.glob(os.path.join(CSRC, "*.cuh"))
+            + glob.glob(os.path.join(CSRC, "*.h"))
             + glob.glob(os.path.join(MEASURE, "*.h")) + [os.path.join(INCLUDE, "hpeel.h")])
 
 

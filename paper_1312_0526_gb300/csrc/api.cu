@@ -14,6 +14,7 @@
 #include <string>
 #include <vector>
 
+#include "held.h"
 #include "host.h"
 #include "kernels.cuh"
 
@@ -25,14 +26,27 @@ thread_local std::string g_last_error;
 
 namespace {
 
-// Small pinned host buffer for the per-round control-block read-back.
-Ctl *pinned_ctl() {
-    thread_local Ctl *p = nullptr;
-    if (!p) {
-        if (cudaMallocHost((void **)&p, sizeof(Ctl)) != cudaSuccess) p = nullptr;
+// What the device writes for the host to read, in pinned memory, one block per
+// thread that calls (held.h): the control blocks read back, the stats of a
+// host-decided small call, and the layer starts of a host-decided peel, read back
+// with its control block for the assignment: the first kHeadLayers + 1 of them (a
+// peel with more rounds reads its table in a second copy).
+constexpr uint32_t kHeadLayers = 1023;
+struct ReadBack {
+    Ctl ctl;
+    LargeCtl large;
+    hpeel_stats stats;
+    uint32_t loff[kHeadLayers + 1];
+};
+ReadBack *make_read_back() {
+    ReadBack *p = nullptr;
+    if (cudaMallocHost((void **)&p, sizeof(ReadBack)) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
     }
     return p;
 }
+ReadBack *read_back() { return Held<ReadBack, make_read_back>::get(); }
 
 struct PeelLayout {
     size_t ctl, params, emit, rec, state, claim, L, pairs, fill, pairs2, fill2, ovf, ovf_count, loff,
@@ -175,27 +189,6 @@ MphfLayout mphf_layout(uint64_t n, uint32_t gamma_milli) {
     return p;
 }
 
-// Where the kernel of a host-decided small call writes its stats.
-hpeel_stats *pinned_stats() {
-    thread_local hpeel_stats *p = nullptr;
-    if (!p) {
-        if (cudaMallocHost((void **)&p, sizeof(hpeel_stats)) != cudaSuccess) p = nullptr;
-    }
-    return p;
-}
-
-// The layer starts of a host-decided peel, read back with its control block
-// for the assignment: the first kHeadLayers + 1 of them (a peel with more
-// rounds reads its table in a second copy).
-constexpr uint32_t kHeadLayers = 1023;
-uint32_t *pinned_loff() {
-    thread_local uint32_t *p = nullptr;
-    if (!p) {
-        if (cudaMallocHost((void **)&p, 4 * (kHeadLayers + 1)) != cudaSuccess) p = nullptr;
-    }
-    return p;
-}
-
 struct PeelOut {
     uint32_t rounds;
     uint64_t n_peeled;
@@ -240,9 +233,10 @@ bool small_route(int mode, const PeelLayout &lay, uint64_t n, uint64_t m, uint32
 // of at most kSmallTries seeds each, the last one's stats in *st.
 hpeel_status run_small_build(const Launch &L, const SmallLaunch &k, SmallArgs a, uint32_t max_tries,
                              hpeel_stats *st) {
-    hpeel_stats *ps = pinned_stats();
-    if (!ps) return fail(HPEEL_ERR_CUDA, "cudaMallocHost of the stats read-back failed");
-    a.stats = ps;
+    ReadBack *rb = read_back();
+    if (!rb) return fail(HPEEL_ERR_CUDA, "cudaMallocHost of the stats read-back failed");
+    const hpeel_stats *ps = &rb->stats;
+    a.stats = &rb->stats;
     const uint64_t seed = a.seed;
     for (uint32_t done = 0; done < max_tries; done += kSmallTries) {
         a.seed = seed + done;
@@ -641,9 +635,9 @@ hpeel_status peel_core_rb(const Launch &L, const PeelIO &io, uint32_t n, uint32_
         ProfScope ps(L, "rounds");
         HP_TRY(launch_round_graph(L, ra));
         if (io.loff_h) {
-            uint32_t *head = pinned_loff();
-            if (!head) return fail(HPEEL_ERR_CUDA, "cudaMallocHost of the layer starts failed");
-            HP_CUDA(cudaMemcpyAsync(head, loff,
+            ReadBack *rb = read_back();
+            if (!rb) return fail(HPEEL_ERR_CUDA, "cudaMallocHost of the layer starts failed");
+            HP_CUDA(cudaMemcpyAsync(rb->loff, loff,
                                     4 * (size_t)std::min(kHeadLayers, lay.max_rounds + 1) + 4,
                                     cudaMemcpyDeviceToHost, L.stream));
         }
@@ -681,7 +675,7 @@ hpeel_status peel_core_rb(const Launch &L, const PeelIO &io, uint32_t n, uint32_
     out->list = Ll;
     if (io.loff_h) {
         if (R <= kHeadLayers && !(tu.host_round_loop || io.host_loop)) {
-            out->loff_h = pinned_loff();
+            out->loff_h = read_back()->loff;
         } else {
             io.loff_h->resize((size_t)R + 1);
             HP_CUDA(cudaMemcpyAsync(io.loff_h->data(), loff, 4 * ((size_t)R + 1),
@@ -752,9 +746,9 @@ hpeel_status peel_core_rb(const Launch &L, const PeelIO &io, uint32_t n, uint32_
 
 hpeel_status peel_core(const Launch &L, const PeelIO &io, uint32_t n, uint32_t m, uint32_t r,
                        char *ws, PeelOut *out) {
-    Ctl *hctl = pinned_ctl();
-    if (!hctl) return fail(HPEEL_ERR_CUDA, "cudaMallocHost of the control read-back failed");
-    return peel_core_rb(L, io, n, m, r, ws, out, hctl);
+    ReadBack *rb = read_back();
+    if (!rb) return fail(HPEEL_ERR_CUDA, "cudaMallocHost of the control read-back failed");
+    return peel_core_rb(L, io, n, m, r, ws, out, &rb->ctl);
 }
 
 // ---------------------------------------------------------------------------
@@ -1291,14 +1285,15 @@ hpeel_status peel_entry(bool general, const uint32_t *d_edges, uint64_t n, uint6
     SmallArgs sa{};
     SmallLaunch sk{};
     if (small_route(0, peel_layout(n, m, r, general), n, m, r, general, (char *)d_ws, &sa, &sk)) {
-        hpeel_stats *ps = pinned_stats();
-        if (!ps) return fail(HPEEL_ERR_CUDA, "cudaMallocHost of the stats read-back failed");
+        ReadBack *rb = read_back();
+        if (!rb) return fail(HPEEL_ERR_CUDA, "cudaMallocHost of the stats read-back failed");
+        const hpeel_stats *ps = &rb->stats;
         sa.edges = d_edges;
         sa.order = d_order;
         sa.claim = d_claim;
         sa.layer_off = d_layer_off;
         sa.max_layers = max_layers;
-        sa.stats = ps;
+        sa.stats = &rb->stats;
         {
             ProfScope prof(L, "small_peel");
             launch_small(L, sk, sa);
@@ -2010,12 +2005,6 @@ cudaError_t capture_large_rounds(cudaStream_t s0, cudaStream_t s1, int sms,
     return e != cudaSuccess ? e : e2;
 }
 
-LargeCtl *pinned_large_ctl() {
-    thread_local LargeCtl *p = nullptr;
-    if (!p && cudaMallocHost((void **)&p, sizeof(LargeCtl)) != cudaSuccess) p = nullptr;
-    return p;
-}
-
 }  // namespace
 
 extern "C" {
@@ -2065,8 +2054,9 @@ hpeel_status hpeel_mphf_build_large(const uint64_t *d_keys, uint64_t n, uint64_t
                         "cudaMallocHost or cudaHostRegister)");
         }
     }
-    LargeCtl *hctl = pinned_large_ctl();
-    if (!hctl) return fail(HPEEL_ERR_CUDA, "cudaMallocHost of the control read-back failed");
+    ReadBack *rb = read_back();
+    if (!rb) return fail(HPEEL_ERR_CUDA, "cudaMallocHost of the control read-back failed");
+    LargeCtl *hctl = &rb->large;
     char *ws = (char *)d_ws;
     LargeCtl *ctl = reinterpret_cast<LargeCtl *>(ws + lay.ctl);
     LargeParams *prm = reinterpret_cast<LargeParams *>(ws + lay.params);
