@@ -10,8 +10,8 @@
 //   hash + AddEdge (sec. 3, 4.1), round 0 scan, rounds with the claims of
 //   round t+1 made by the deletions of round t (sec. 4.2; same scheme as the
 //   single-graph path), the canonical order (layers ascending by round, edge
-//   ids ascending inside a layer, 2-core edges last) by a stable counting pass, and optionally the MWHC g values (sec. 3, layers last to
-//   first).
+//   ids ascending inside a layer, 2-core edges last) by a stable counting pass,
+//   and optionally the MWHC g values (sec. 3, layers last to first).
 // A bucket's state lives in shared memory when it fits: vertex records of 32
 // bits (degree in the low 16, sum of incident local edge ids mod 2^16 in the
 // high 16; a bucket in shared memory has far fewer than 2^16 edges, so the

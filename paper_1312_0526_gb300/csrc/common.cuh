@@ -217,20 +217,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
 // degree 1 with its last edge claimed (round 0 scan, or the fall from 2 to 1).
 constexpr uint32_t kMark = 0x80000000u;
 
-// Warp-aggregated append: every lane of the warp calls this (convergent);
-// lanes with pred get consecutive slots of list, one atomicAdd per warp.
-__device__ __forceinline__ void warp_append(uint32_t *cursor, uint32_t *list, bool pred,
-                                            uint32_t value) {
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t ballot = __ballot_sync(0xFFFFFFFFu, pred);
-    if (ballot == 0) return;
-    uint32_t base = 0;
-    const uint32_t leader = __ffs(ballot) - 1;
-    if (lane == leader) base = atomicAdd(cursor, (uint32_t)__popc(ballot));
-    base = __shfl_sync(0xFFFFFFFFu, base, leader);
-    if (pred) list[base + __popc(ballot & ((1u << lane) - 1u))] = value;
-}
-
 // ---- edge records ------------------------------------------------------
 // Edge e: one uint4 {v_0, v_1, v_2, claim} for r <= 3 (v_2 = 0 when r = 2),
 // two uint4 {v_0..v_3}, {claim, 0, 0, 0} for r = 4.
@@ -378,45 +364,6 @@ __device__ __forceinline__ void unrotate(const uint32_t (&v)[4], uint32_t h, uin
     for (int k = R; k < 4; k++) p[k] = 0u;
 }
 
-// Block-aggregated append: every thread of the block calls this (it holds
-// barriers) with K candidates; the block reserves all its slots with a single
-// atomicAdd, so the shared cursor sees one atomic per K * blockDim items.
-// The order of the appended values inside the list is unspecified.
-template <int K, int THREADS>
-__device__ __forceinline__ void block_append(uint32_t *cursor, uint32_t *list, const bool (&pred)[K],
-                                             const uint32_t (&val)[K]) {
-    __shared__ uint32_t warp_base[THREADS / 32];
-    __shared__ uint32_t block_base;
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    uint32_t cnt = 0;
-#pragma unroll
-    for (int k = 0; k < K; k++) cnt += pred[k] ? 1u : 0u;
-    uint32_t x = cnt;  // inclusive warp scan
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, d);
-        if (lane >= (uint32_t)d) x += y;
-    }
-    if (lane == 31) warp_base[warp] = x;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t s = 0;
-#pragma unroll
-        for (int w = 0; w < THREADS / 32; w++) {
-            const uint32_t c = warp_base[w];
-            warp_base[w] = s;
-            s += c;
-        }
-        block_base = s ? atomicAdd(cursor, s) : 0u;
-    }
-    __syncthreads();
-    uint32_t pos = block_base + warp_base[warp] + x - cnt;
-#pragma unroll
-    for (int k = 0; k < K; k++)
-        if (pred[k]) list[pos++] = val[k];
-    __syncthreads();
-}
-
 // Per-warp staging buffer in shared memory for list appends: lanes push
 // values (warp-synchronous), and the warp reserves space in the global list
 // with one atomicAdd per CAP values (flush when full and at the end), so the
@@ -450,31 +397,5 @@ struct WarpStage {
         __syncwarp();
     }
 };
-
-// Block-aggregated reservation of one slot per thread with pred: returns the
-// slot (unspecified order) for those threads; one atomicAdd per block call.
-template <int THREADS>
-__device__ __forceinline__ uint32_t block_reserve(uint32_t *cursor, bool pred) {
-    __shared__ uint32_t warp_base[THREADS / 32];
-    __shared__ uint32_t block_base;
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint32_t ballot = __ballot_sync(0xFFFFFFFFu, pred);
-    if (lane == 0) warp_base[warp] = __popc(ballot);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t s = 0;
-#pragma unroll
-        for (int w = 0; w < THREADS / 32; w++) {
-            const uint32_t c = warp_base[w];
-            warp_base[w] = s;
-            s += c;
-        }
-        block_base = s ? atomicAdd(cursor, s) : 0u;
-    }
-    __syncthreads();
-    const uint32_t pos = block_base + warp_base[warp] + __popc(ballot & ((1u << lane) - 1u));
-    __syncthreads();
-    return pos;
-}
 
 }  // namespace hp

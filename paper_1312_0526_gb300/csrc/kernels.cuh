@@ -233,7 +233,7 @@ struct SortedBufs {
     uint32_t *fill2;
     uint2 *claims;
 };
-// min_edges: 0 automatic (n / 24), 0xFFFFFFFF never; b: the incidence
+// min_edges: 0 automatic (n / 20), 0xFFFFFFFF never; b: the incidence
 // build's bucket plan (its vertex chunks are reused).
 SortedPlan sorted_plan(uint64_t n, uint64_t m, uint32_t r, const BucketPlan &b, uint32_t min_edges,
                        int sms);
