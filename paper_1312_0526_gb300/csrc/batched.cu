@@ -604,10 +604,11 @@ void launch_batch_g_offsets(const Launch &L, const uint64_t *off, uint32_t B, ui
 // shape for all sizes leaves half the keys of a lognormal workload in the
 // global regions (2.01e8 keys in 65,536 buckets: 14.9 ms at 256 threads x 6
 // blocks, the best single shape).  Rates of uniform buckets (keys per us and
-// SM, with g values) at the shape chosen and at the next best: 200 keys 119 /
-// 108, 1000 182 / 159, 1500 158 / 147, 2000 152 / 141, 3500 147 / 145, 4000
-// 131 / 130, 6000 118 / 112, 8000 107 / 104, 12000 102 / 97, 24000 95 / 91,
-// 60000 (global regions) 33 / 25 (before one warp took the small layers).
+// SM, with g values) at the class's shape and at the best other of 24: 200 keys
+// 140 / 154 (128 threads x 16), 500 191 / 211 (128 x 16), 1000 189 / 226 (128 x
+// 12), 1500 197 / 200, 2000 188 / 174, 3500 177 / 174, 4000 160 / 156, 6000 143 /
+// 140, 8000 120 / 120, 12000 114 / 113, 24000 101 / 102.  (The classes were chosen
+// before one warp took the small layers, when each was the best at its sizes.)
 struct BatchClass {
     uint32_t threads, ctas;
     bool verts;   // takes buckets whose vertices fit beside their state, or

@@ -9,8 +9,9 @@
 // cluster's own edges, one shared-memory atomic per deleted incidence and one
 // hardware barrier (barrier.cluster between blocks: no spinning, and the
 // hardware starts the blocks of a cluster together): 0.35 us per round at
-// n = 1e3, 0.9 us at 12,000, 1.9 us at 1e5.  MPHF build of 1009 keys 1115 ->
-// 60 us (kernel 28 us), peel of 1e5 edges 930 -> 190 us (kernel 166 us).
+// n = 1e3, 0.9 us at 12,000, 1.9 us at 1e5.  MPHF build of 1009 keys 810-1000 ->
+// 56-63 us (kernel 31 us where the first seed peels), hash and peel of 1e5 edges
+// 830-910 -> 183-198 us (kernel of the peel 168 us).
 //
 // Layout.  Block c of the cluster owns epc consecutive edges (their vertices
 // and claim words) and every vertex whose 512-vertex group is c modulo the
@@ -892,7 +893,8 @@ const void *small_fn(int mode, uint32_t r, bool gen, bool solo, uint32_t ept) {
 
 // Edges per thread of the one-block forms (kernel time per peel / MPHF build):
 // n = 1009 with one edge per thread 18.6 / 27.8 us, with four 32.9 / 55; n =
-// 4000 with four 45 / 82 us, with sixteen 60 / 74.
+// 4000 with four 45 / 82 us, with sixteen 60 / 74 (before claims were counted,
+// which takes 1-4 % more).
 constexpr uint32_t kSmOnePer = 1024, kSmFourPer = 4096;
 // Shape of a launch: blocks (a power of two), edges per thread, edges and
 // vertex slots per block, threads, dynamic shared memory.
