@@ -534,8 +534,8 @@ hpeel_status hpeel_sf_lookup(const uint64_t *d_keys, uint64_t nq, uint64_t seed,
 typedef struct hpeel_batch_tuning {
     uint32_t threads;      /* threads per block (multiple of 32, 64..1024; 0: 256).
                               threads, ctas_per_sm and smem_bytes all 0: one launch
-                              per size class of the buckets, each with a shape that
-                              suits it; any of them given: one launch of that shape */
+                              per size class that B buckets can fill, each with a
+                              shape that suits it; any of them given: one launch of that shape */
     uint32_t ctas_per_sm;  /* blocks per SM (grid = SMs x this; 0: 2) */
     uint32_t smem_bytes;   /* shared memory per block for bucket state (0: the SM's
                               shared memory split between the blocks); buckets
